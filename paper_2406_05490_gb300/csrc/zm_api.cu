@@ -222,7 +222,7 @@ void zm_destroy(zm_ctx *c)
         c->batch = nullptr;
         c->y0 = c->ya = c->yb = c->u = c->phi = c->q = nullptr;
     }
-    void *bufs[] = {c->y0, c->ya, c->yb, c->u, c->phi, c->q, c->nrm, c->src, c->part,
+    void *bufs[] = {c->y0, c->ya, c->yb, c->u, c->phi, c->q, c->nrm, c->src, c->src_far, c->part,
                     c->fa, c->fb, c->tw1, c->tw2, c->twl1, c->twl2, c->twh, c->err, c->flag};
     for (void *b : bufs)
         if (b) cudaFree(b);
@@ -326,8 +326,9 @@ int zm_create(const zm_mesh *mesh, double atwood, double g, double mu, double de
         c->tiling = make_tiling(G);
         const size_t slots = (size_t)c->tiling.ntiles * c->tiling.ts;
         c->plan = plan_br(G, c->tiling, sms);
-        c->src_bytes = slots * kRec64 * sizeof(double);
-        ok = alloc(&c->src, c->src_bytes) &&
+        const bool dw = brdw_mesh(G);
+        c->src_bytes = dw ? brdw_near_bytes(G) : slots * kRec64 * sizeof(double);
+        ok = alloc(&c->src, c->src_bytes) && (!dw || alloc((void **)&c->src_far, brdw_far_bytes(G))) &&
              alloc((void **)&c->part, (size_t)c->plan.nsplit * 3 * N * sizeof(double));
         // padding slots of edge tiles stay zero for good: zero strength, no contribution
         if (ok) ok = cudaMemset(c->src, 0, c->src_bytes) == cudaSuccess;

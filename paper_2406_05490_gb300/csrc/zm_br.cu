@@ -13,12 +13,12 @@
 // memory.  Split partial sums go to a [nsplit][3][N] workspace reduced in a fixed order by the
 // reduction kernel, which keeps results deterministic.
 //
-// This file holds the FP64 variant (every operation in FP64; the kernel (|r|^2 + delta^2)^(-3/2)
-// from the hardware reciprocal-square-root estimate and one second-order correction, see
-// dev::rsqrt_cube) -- the plain per-instance comparator -- and its allocation-free form; the
-// FP32-compensated variant is in zm_br32.cu.  Per pair: 21 FP64 instructions (3 differences,
-// 3 FMAs for |r|^2 + delta^2, 6 for the kernel, 6 for the cross product, 3 accumulations) and
-// one MUFU operation, for 26 counted flops.
+// This file holds the plain FP64 variant (every operation in FP64; the kernel (|r|^2 +
+// delta^2)^(-3/2) from the hardware reciprocal-square-root estimate and one second-order
+// correction, see dev::rsqrt_cube), which meshes below 56^2 nodes and the allocation-free entry
+// point use; larger FP64 meshes take zm_brdw.cu, the FP32-compensated variant is in zm_br32.cu.
+// Per pair: 21 FP64 instructions (3 differences, 3 FMAs for |r|^2 + delta^2, 6 for the kernel, 6 for
+// the cross product, 3 accumulations) and one MUFU operation, for 26 counted flops.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -153,29 +153,18 @@ Tiling make_tiling(const Geom &g) { return make_tiling_shape(g, kTile1, kTile2);
 
 BrPlan plan_br(const Geom &g, const Tiling &t, int sm_count)
 {
+    if (brdw_mesh(g)) return plan_brdw(g, sm_count);
+    // one-warp target blocks and, as far as the GPU is not full, sources split below a tile: up to
+    // 16 slices of 16 sources (a 32^2 mesh then runs 1024 one-warp CTAs, ~7 per SM)
     BrPlan p;
-    p.tpb = kTpb64;
+    p.tpb = kTpb64s;
     p.r = kR64;
-    p.qsplit = 1;
     const int want = 4 * sm_count;  // about four resident CTAs per SM over the grid
     p.ntb = (g.N + p.tpb * p.r - 1) / (p.tpb * p.r);
-    if ((long long)p.ntb * t.ntiles < want) {
-        // small mesh: one-warp target blocks and sources split below a tile
-        p.tpb = kTpb64s;
-        p.ntb = (g.N + p.tpb * p.r - 1) / (p.tpb * p.r);
-        p.qsplit = 1;
-        // up to 16 slices of 16 sources: a 32^2 mesh then runs 1024 one-warp CTAs (~7 per SM)
-        while (p.qsplit < 16 && (long long)p.ntb * t.ntiles * p.qsplit < want) p.qsplit *= 2;
-        if (p.qsplit > 1) {
-            p.tiles_per_split = 1;
-            p.nsplit = t.ntiles * p.qsplit;
-            return p;
-        }
-    }
-    int ns = (want + p.ntb - 1) / p.ntb;
-    ns = std::max(1, std::min(ns, t.ntiles));
-    p.tiles_per_split = (t.ntiles + ns - 1) / ns;
-    p.nsplit = (t.ntiles + p.tiles_per_split - 1) / p.tiles_per_split;
+    p.qsplit = 1;
+    while (p.qsplit < 16 && (long long)p.ntb * t.ntiles * p.qsplit < want) p.qsplit *= 2;
+    p.tiles_per_split = 1;
+    p.nsplit = t.ntiles * p.qsplit;
     return p;
 }
 
@@ -183,18 +172,14 @@ int launch_br(zm_ctx *c, const double *y)
 {
     if (!y || !c->src || !c->part) return set_error(ZM_ERR_INVALID, "Birkhoff-Rott pass: missing buffer");
     const Geom &g = c->geom;
+    if (brdw_mesh(g)) return launch_brdw(c, y);
     const BrPlan &p = c->plan;
     dim3 grid(p.ntb, p.nsplit);
     cudaEvent_t ev = nullptr;
     prof_begin(c, ZM_K_BR, &ev);
-    if (p.tpb == kTpb64s)
-        br64_kernel<kTpb64s, kR64, kTile1 * kTile2><<<grid, kTpb64s, 0, c->stream>>>(
-            g.N, y, static_cast<const double *>(c->src), c->tiling.ntiles, p.tiles_per_split,
-            p.qsplit, c->delta * c->delta, c->part, c->err);
-    else
-        br64_kernel<kTpb64, kR64, kTile1 * kTile2><<<grid, kTpb64, 0, c->stream>>>(
-            g.N, y, static_cast<const double *>(c->src), c->tiling.ntiles, p.tiles_per_split,
-            p.qsplit, c->delta * c->delta, c->part, c->err);
+    br64_kernel<kTpb64s, kR64, kTile1 * kTile2><<<grid, kTpb64s, 0, c->stream>>>(
+        g.N, y, static_cast<const double *>(c->src), c->tiling.ntiles, p.tiles_per_split, p.qsplit,
+        c->delta * c->delta, c->part, c->err);
     prof_end(c, ZM_K_BR, ev);
     c->prof.acc.pairs += (int64_t)g.N * (int64_t)g.N;
     return cuda_check(cudaGetLastError(), "Birkhoff-Rott kernel launch");

@@ -147,7 +147,7 @@ struct zm_ctx {
     void *src;
     size_t src_bytes;
     double *part;  // FP64: [nsplit][3][N]; FP32C: [ctas * kseg][3][512]
-    float *src_far;   // FP32C far records
+    float *src_far;   // FP64 on larger meshes: tile infos and far records (zm_brdw.cu)
     float4 *tinfo;    // FP32C per-tile bounding sphere: centre, radius
     zm::Br32Plan plan32;
 
@@ -201,6 +201,14 @@ Tiling make_tiling(const Geom &g);  // 16 x 16 patches
 // tp1 x tp2 patches (tp1 * tp2 = 256 slots, both powers of two)
 Tiling make_tiling_shape(const Geom &g, int tp1, int tp2);
 int launch_br(zm_ctx *c, const double *y);  // FP64 path (then launch_reduce)
+
+// ---- the same for meshes of at least 48^2 nodes: far pairs in FP32 pairs (zm_brdw.cu) --------------
+bool brdw_mesh(const Geom &g);
+BrPlan plan_brdw(const Geom &g, int sm_count);
+size_t brdw_near_bytes(const Geom &g);
+size_t brdw_far_bytes(const Geom &g);
+int launch_geometry_dw(zm_ctx *c, const double *y, double pref);
+int launch_brdw(zm_ctx *c, const double *y);
 
 // ---- FP32C Birkhoff-Rott kernel over a batch of interfaces (zm_br32.cu) ----------------------------
 int br32_occupancy();  // resident CTAs per SM of the batched kernel
@@ -302,6 +310,7 @@ static __device__ __noinline__ bool fail(long long i, int site)
 int bounds_api(unsigned int *, long long *, int *, int);
 int bounds_batch(unsigned int *, long long *, int *, int);
 int bounds_br(unsigned int *, long long *, int *, int);
+int bounds_brdw(unsigned int *, long long *, int *, int);
 int bounds_br32(unsigned int *, long long *, int *, int);
 int bounds_br32tc(unsigned int *, long long *, int *, int);
 int bounds_fft(unsigned int *, long long *, int *, int);

@@ -124,7 +124,11 @@ int launch_geometry(zm_ctx *c, const double *y)
             prof_end(c, ZM_K_GEOMETRY, ev);
             prof_begin(c, ZM_K_GEOMETRY, &ev);
         }
-        geometry_kernel<kGeoFp64><<<grid, kTpb, 0, c->stream>>>(g, c->tiling, y, pref, c->g, c->src,
+        if (brdw_mesh(g)) {
+            const int rc = launch_geometry_dw(c, y, pref);
+            if (rc) return rc;
+        } else
+            geometry_kernel<kGeoFp64><<<grid, kTpb, 0, c->stream>>>(g, c->tiling, y, pref, c->g, c->src,
                                                               c->q, nullptr);
     }
     prof_end(c, ZM_K_GEOMETRY, ev);

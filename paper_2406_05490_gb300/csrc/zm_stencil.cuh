@@ -53,6 +53,40 @@ __device__ __forceinline__ double diff2(const double v[5], double inv12dx2)
 //   kGeoLow: unit normal.
 constexpr int kGeoFp64 = 0, kGeoFp32c = 1, kGeoLow = 2;
 
+// Tangents a1 = D1 z, a2 = D2 z at node (i, j).
+__device__ __forceinline__ void tangents(const Geom &g, int i, int j, const double *__restrict__ z, double a1[3],
+                                         double a2[3])
+{
+    double v[5];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        line5(z + (size_t)c * g.N, i, j, 0, g, c == 0 ? g.L1 : 0.0, v);
+        a1[c] = diff1(v, g.i12a);
+        line5(z + (size_t)c * g.N, i, j, 1, g, c == 1 ? g.L2 : 0.0, v);
+        a2[c] = diff1(v, g.i12b);
+    }
+}
+
+// High order at node p: the scaled sheet strength gamma' = (dx1 dx2 / 4 pi) (w1 a2 - w2 a1) in gm;
+// returns q.
+__device__ __forceinline__ double geometry_strength(const Geom &g, int p, const double *__restrict__ y, double pref,
+                                                    double grav, double gm[3])
+{
+    const int i = p / g.n2, j = p - (p / g.n2) * g.n2;
+    double a1[3], a2[3];
+    tangents(g, i, j, y, a1, a2);
+    const double *w = y + 3 * (size_t)g.N;
+    const double h11 = a1[0] * a1[0] + a1[1] * a1[1] + a1[2] * a1[2];
+    const double h12 = a1[0] * a2[0] + a1[1] * a2[1] + a1[2] * a2[2];
+    const double h22 = a2[0] * a2[0] + a2[1] * a2[1] + a2[2] * a2[2];
+    const double det = h11 * h22 - h12 * h12;
+    const double w1 = w[p], w2 = w[(size_t)g.N + p];
+    const double quad = h22 * w1 * w1 - 2.0 * h12 * w1 * w2 + h11 * w2 * w2;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) gm[c] = pref * (w1 * a2[c] - w2 * a1[c]);
+    return grav * y[2 * (size_t)g.N + p] + 0.125 * quad / det;
+}
+
 template <int kKind>
 __device__ __forceinline__ void geometry_point(const Geom &g, const Tiling &t, int p,
                                                const double *__restrict__ y, double pref,
@@ -63,42 +97,29 @@ __device__ __forceinline__ void geometry_point(const Geom &g, const Tiling &t, i
 {
     if (!ZM_IDX_OK(p, g.N)) return;
     const int i = p / g.n2, j = p - (p / g.n2) * g.n2;
-    const double *z = y, *w = y + 3 * (size_t)g.N;
-    const double i12a = g.i12a, i12b = g.i12b;
-
-    double a1[3], a2[3], v[5];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        line5(z + (size_t)c * g.N, i, j, 0, g, c == 0 ? g.L1 : 0.0, v);
-        a1[c] = diff1(v, i12a);
-        line5(z + (size_t)c * g.N, i, j, 1, g, c == 1 ? g.L2 : 0.0, v);
-        a2[c] = diff1(v, i12b);
-    }
-    const double h11 = a1[0] * a1[0] + a1[1] * a1[1] + a1[2] * a1[2];
-    const double h12 = a1[0] * a2[0] + a1[1] * a2[1] + a1[2] * a2[2];
-    const double h22 = a2[0] * a2[0] + a2[1] * a2[1] + a2[2] * a2[2];
-    const double det = h11 * h22 - h12 * h12;
-    const double w1 = w[p], w2 = w[(size_t)g.N + p];
-    const double z3 = z[2 * (size_t)g.N + p];
-    const double quad = h22 * w1 * w1 - 2.0 * h12 * w1 * w2 + h11 * w2 * w2;
-
+    const double *z = y;
     if (kKind == kGeoLow) {
+        double a1[3], a2[3];
+        tangents(g, i, j, z, a1, a2);
+        const double *w = y + 3 * (size_t)g.N;
+        const double h11 = a1[0] * a1[0] + a1[1] * a1[1] + a1[2] * a1[2];
+        const double h12 = a1[0] * a2[0] + a1[1] * a2[1] + a1[2] * a2[2];
+        const double h22 = a2[0] * a2[0] + a2[1] * a2[1] + a2[2] * a2[2];
+        const double w1 = w[p], w2 = w[(size_t)g.N + p];
+        const double quad = h22 * w1 * w1 - 2.0 * h12 * w1 * w2 + h11 * w2 * w2;
         // unit normal; |a1 x a2|^2 = det (Lagrange's identity) also gives 1/det
         const double nx = a1[1] * a2[2] - a1[2] * a2[1];
         const double ny = a1[2] * a2[0] - a1[0] * a2[2];
         const double nz = a1[0] * a2[1] - a1[1] * a2[0];
         const double il = dev::rsqrt_nr(nx * nx + ny * ny + nz * nz);
-        q[p] = grav * z3 + 0.125 * quad * (il * il);
+        q[p] = grav * z[2 * (size_t)g.N + p] + 0.125 * quad * (il * il);
         nrm[p] = nx * il;
         nrm[(size_t)g.N + p] = ny * il;
         nrm[2 * (size_t)g.N + p] = nz * il;
         return;
     }
-    q[p] = grav * z3 + 0.125 * quad / det;
-    // scaled sheet strength gamma' = (dx1 dx2 / 4 pi) (w1 a2 - w2 a1)
     double gm[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) gm[c] = pref * (w1 * a2[c] - w2 * a1[c]);
+    q[p] = geometry_strength(g, p, y, pref, grav, gm);
 
     const int ti = i / t.tp1, tj = j / t.tp2;
     const size_t tile = (size_t)ti * t.nt2 + tj;
