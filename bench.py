@@ -460,9 +460,14 @@ def bench_low_order(zm, torch, inputs, flush, nl, steps, warmup, df64, fp64_tflo
             inst, kind = fp64_inst_record().get(k, (None, None))
             if kind == "by_side":
                 inst = inst.get(nl)  # counted per mesh side; None for a side not counted
-            kern[k]["fp64_inst_per_point"] = inst
-            kern[k]["fp64_pipe_frac"] = (inst * pts / (t * 1e-3) / (fp64_tflops * 1e12 / 2)
-                                         if inst and t > 0 else None)
+            if k == "fft":  # integer transforms: all executed thread instructions, of the issue rate
+                kern[k]["inst_per_point"] = inst
+                kern[k]["issue_frac"] = (inst / 32 * pts / (t * 1e-3) / issue_rate
+                                         if inst and issue_rate and t > 0 else None)
+            else:
+                kern[k]["fp64_inst_per_point"] = inst
+                kern[k]["fp64_pipe_frac"] = (inst * pts / (t * 1e-3) / (fp64_tflops * 1e12 / 2)
+                                             if inst and t > 0 else None)
     step_bytes = 3 * sum(LOW_BYTES.values()) * pts
     return {"precision": "double-word (FP32 pairs)" if df64 else "fp64", "points": pts,
             "steps": steps, "steps_per_s": steps / (msl * 1e-3), "ms_per_step": msl / steps,
@@ -832,7 +837,7 @@ def run_gb300(args):
         # low order (FFT Riesz velocity): 1024^2 (the low-vs-high configuration), FP64 and
         # double-word; 4096^2, the largest power-of-two side below the paper's 4864^2 mesh
         issue_rate = sm_count * 4 * clk_mhz * 1e6  # warp instructions per second at one per scheduler per clock
-        extras["low_order_1024"] = bench_low_order(zm, torch, inputs, flush, 1024, 10, 3, False, fp64_peak)
+        extras["low_order_1024"] = bench_low_order(zm, torch, inputs, flush, 1024, 10, 3, False, fp64_peak, issue_rate)
         extras["low_order_1024_df64"] = bench_low_order(zm, torch, inputs, flush, 1024, 10, 3, True, issue_rate=issue_rate)
         # the high-order half of the low-vs-high configuration: the same 8-mode interface
         # (amplitude 0.02, A = 0.7) at 512^2, FP32C all-pairs sum, 10 RK3 steps
@@ -853,10 +858,10 @@ def run_gb300(args):
             "br_frac_of_fp32_peak": FLOPS_PER_PAIR * nh**4 / (br_h * 1e-3) / 1e12 / peak,
             "peak_basis": "measured FP32 FMA probe (as the headline roofline)",
             "kernel_ms_per_step": {k: v / kh for k, v in profh["ms"].items()}}
-        extras["low_order_4096"] = bench_low_order(zm, torch, inputs, flush, 4096, 3, 1, False, fp64_peak)
+        extras["low_order_4096"] = bench_low_order(zm, torch, inputs, flush, 4096, 3, 1, False, fp64_peak, issue_rate)
         extras["low_order_4096_df64"] = bench_low_order(zm, torch, inputs, flush, 4096, 5, 2, True, issue_rate=issue_rate)
         # the paper's single-GPU low-order mesh: 4864^2 = (19 x 256)^2, FP64 (radix-19 stage)
-        extras["low_order_4864"] = bench_low_order(zm, torch, inputs, flush, 4864, 3, 1, False, fp64_peak)
+        extras["low_order_4864"] = bench_low_order(zm, torch, inputs, flush, 4864, 3, 1, False, fp64_peak, issue_rate)
         extras["low_order_4864_df64"] = bench_low_order(zm, torch, inputs, flush, 4864, 5, 2, True, issue_rate=issue_rate)
         # 32^2 single-mode FP64 (launch bound)
         zs, wsn = inputs.single_mode(32)

@@ -155,6 +155,8 @@ struct zm_ctx {
     // factor M of each side, twl1, twl2 for the whole side L = R M when R > 1 (else null)
     double2 *fa, *fb, *tw1, *tw2, *twl1, *twl2;
     double2 *twh;  // double word, both sides powers of two: half table of W_{n2/2} (else null)
+    void *fmult;   // FP64 low/medium order: the Riesz multipliers over a quarter of the spectrum
+    int *fexp;     // FP64 low/medium order: the FFT passes' exponents (two maxima, then per CTA)
 
     int *err;   // device status word (zm::kErr*)
     int *flag;  // device scratch flag (finite check)
