@@ -21,8 +21,8 @@
 //
 // Cutoff (paper Sec. 3.2.2 CutoffBRSolver: only sources within a 3D distance of the target).
 // With a cutoff c, the tile spheres classify each (target tile, source tile): entirely beyond c
-// (skipped: no copy, no work), entirely within c (the paths above), or straddling c (the near
-// path with a per-pair test |r|^2 <= c^2 on the FP32 hi/lo difference, exact to about 2^-22 in
+// (skipped: no copy, no work), entirely within c (the paths above), or straddling c (the same two
+// paths with a per-pair test |r|^2 <= c^2 on the FP32 hi/lo difference, exact to about 2^-22 in
 // the distance; a pair that close to c may fall either way).  Compact tiles of the
 // mesh act as the cell list.  A relative margin of 1e-4 on c keeps the sphere decisions on the
 // safe side of every pair decision.
@@ -67,6 +67,113 @@ struct Unit {
     int src;   // source tile
     int far;
 };
+
+// Far pair terms of one source tile (stage `s`) for this thread's kR targets (near-record row pointer
+// tr0, kT apart); cs: the source tile's centre.
+// kMask: the tile pair straddles the cutoff; only pairs with |r|^2 <= c2 count, thr = c2 + delta^2.  The
+// Gram form decides, except for pairs closer to the cutoff than its own error, which is below
+// 11 2^-24 (|s| + |t|)^2 (the roundings of s, t, their squares and the four sums) <= 2^-19 (|t|^2 +
+// radius^2); about one pair in 10^5 is as close.  Those are decided as near_tile does, on the FP32
+// hi/lo difference (source record src_near), and their q is moved to their side of thr.  (The near
+// form for all of these pairs, 23 FP32 operations and the mask against 12 and the mask: 512 x 512,
+// cutoff 0.2: 9.9 against 7.3 ms per evaluation.)
+template <bool kMask>
+__device__ __forceinline__ void far_tile(const float *s, const float4 cs, const float *__restrict__ tr0,
+                                         const float *__restrict__ src_near, float thr, float c2, float mult,
+                                         long long (*acc)[kR][kT], int tid)
+{
+    u64 m2x[kR], m2y[kR], m2z[kR], bb[kR];
+    u64 ax[kR], ay[kR], az[kR], gxs[kR], gys[kR], gzs[kR];
+    float bmax = 0.0f;
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+        const float *tr = tr0 + r * kT;
+        const float tx = (__ldg(tr) - cs.x) + __ldg(tr + 3 * kTs);
+        const float ty = (__ldg(tr + kTs) - cs.y) + __ldg(tr + 4 * kTs);
+        const float tz = (__ldg(tr + 2 * kTs) - cs.z) + __ldg(tr + 5 * kTs);
+        m2x[r] = pack2(-2.0f * tx, -2.0f * tx);
+        m2y[r] = pack2(-2.0f * ty, -2.0f * ty);
+        m2z[r] = pack2(-2.0f * tz, -2.0f * tz);
+        const float b1 = fmaf(tx, tx, fmaf(ty, ty, tz * tz));
+        bb[r] = pack2(b1, b1);
+        if (kMask) bmax = r ? fmaxf(bmax, b1) : b1;
+        ax[r] = ay[r] = az[r] = gxs[r] = gys[r] = gzs[r] = 0ull;
+    }
+    const u64 nthr = pack2(-thr, -thr);
+    const float eps = (bmax + cs.w * cs.w) * 1.9073486328125e-6f;  // 2^-19 (|t|^2 + radius^2)
+    const u64 *s2 = reinterpret_cast<const u64 *>(s);  // row k, sources (2m, 2m+1)
+#pragma unroll kFarUnroll
+    for (int m = 0; m < kTs / 2; ++m) {
+        const u64 sx = s2[m], sy = s2[kTs / 2 + m], sz = s2[kTs + m], sa = s2[3 * (kTs / 2) + m];
+        const u64 gx = s2[2 * kTs + m], gy = s2[5 * (kTs / 2) + m], gz = s2[3 * kTs + m];
+        const u64 mx = s2[7 * (kTs / 2) + m], my = s2[4 * kTs + m], mz = s2[9 * (kTs / 2) + m];
+        auto q_of = [&](int r) {
+            return ffma2(sx, m2x[r], ffma2(sy, m2y[r], ffma2(sz, m2z[r], fadd2(sa, bb[r]))));
+        };
+        u64 qm[kR];
+        if (kMask) {
+            float close = eps;
+#pragma unroll
+            for (int r = 0; r < kR; ++r) {
+                qm[r] = q_of(r);
+                float da, db;
+                unpack2(fadd2(qm[r], nthr), da, db);
+                close = fminf(close, fminf(fabsf(da), fabsf(db)));
+            }
+            if (close < eps) {
+#pragma unroll 1
+                for (int k = 0; k < 2 * kR; ++k) {
+                    const int r = k >> 1;
+                    const float *a = src_near + 2 * m + (k & 1), *b = tr0 + r * kT;
+                    const float rx = (a[0] - b[0]) + (a[3 * kTs] - b[3 * kTs]);
+                    const float ry = (a[kTs] - b[kTs]) + (a[4 * kTs] - b[4 * kTs]);
+                    const float rz = (a[2 * kTs] - b[2 * kTs]) + (a[5 * kTs] - b[5 * kTs]);
+                    const bool in = fmaf(rx, rx, fmaf(ry, ry, rz * rz)) <= c2;
+                    const float above = __uint_as_float(__float_as_uint(thr) + 1u);
+#pragma unroll
+                    for (int t = 0; t < kR; ++t) {
+                        float q[2];
+                        unpack2(qm[t], q[0], q[1]);
+                        const float v = q[k & 1];
+                        if (t == r && fabsf(v - thr) < eps)
+                            (k & 1 ? q[1] : q[0]) = in ? fminf(v, thr) : fmaxf(v, above);
+                        qm[t] = pack2(q[0], q[1]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+            const u64 q = kMask ? qm[r] : q_of(r);
+            u64 iq = rsqrt2(q);
+            if (kMask) {
+                float qa, qb, ya, yb;
+                unpack2(q, qa, qb);
+                unpack2(iq, ya, yb);
+                iq = pack2(qa <= thr ? ya : 0.0f, qb <= thr ? yb : 0.0f);
+            }
+            const u64 kk = fmul2(fmul2(iq, iq), iq);
+            ax[r] = ffma2(kk, mx, ax[r]);
+            ay[r] = ffma2(kk, my, ay[r]);
+            az[r] = ffma2(kk, mz, az[r]);
+            gxs[r] = ffma2(kk, gx, gxs[r]);
+            gys[r] = ffma2(kk, gy, gys[r]);
+            gzs[r] = ffma2(kk, gz, gzs[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+        // t = -m2 / 2 exactly (both lanes of m2 hold -2 t)
+        const float tx = -0.25f * sum2(m2x[r]), ty = -0.25f * sum2(m2y[r]), tz = -0.25f * sum2(m2z[r]);
+        const float bx = sum2(gxs[r]), by = sum2(gys[r]), bz = sum2(gzs[r]);
+        const float vx = sum2(ax[r]) - fmaf(ty, bz, -tz * by);
+        const float vy = sum2(ay[r]) - fmaf(tz, bx, -tx * bz);
+        const float vz = sum2(az[r]) - fmaf(tx, by, -ty * bx);
+        acc[0][r][tid] += __float2ll_rn(vx * mult);
+        acc[1][r][tid] += __float2ll_rn(vy * mult);
+        acc[2][r][tid] += __float2ll_rn(vz * mult);
+    }
+}
 
 // kCut: some interface of the batch sums within a cutoff, so straddling tile pairs (masked
 // near path) can occur; without it that path is compiled out.
@@ -127,13 +234,13 @@ __global__ void __launch_bounds__(kT, ZM_BR32_MINB)
             if (I.cutoff > 0.0) {
                 const float c = (float)I.cutoff;
                 if (D - a.w - b.w > c * 1.0001f) continue;          // every pair beyond c
-                if (D + a.w + b.w >= c * 0.9999f) path = 2;         // straddles c: masked near
+                if (D + a.w + b.w >= c * 0.9999f) path = path ? 3 : 2;  // straddles c: masked far or near
             }
             unit[buf].inst = p_inst;
             unit[buf].tile = p_tile;
             unit[buf].src = S;
             unit[buf].far = path;
-            if (path == 1) {
+            if (path & 1) {
                 const float *rec = I.far_rec + (size_t)S * kRec32F * kTs;
                 dev::mbar_expect_tx(&bar[buf], kStageRows * kTs * sizeof(float));
                 dev::tma_copy_1d(stage[buf], rec, 4 * kTs * sizeof(float), &bar[buf]);
@@ -209,54 +316,11 @@ __global__ void __launch_bounds__(kT, ZM_BR32_MINB)
         if (ok) {
             const float *s = stage[b];
             if (un.far == 1) {
-                // ---- far path ------------------------------------------------------------
-                const float4 cs = insts[c_inst].tinfo[un.src];
-                u64 m2x[kR], m2y[kR], m2z[kR], bb[kR];
-                u64 ax[kR], ay[kR], az[kR], gxs[kR], gys[kR], gzs[kR];
-#pragma unroll
-                for (int r = 0; r < kR; ++r) {
-                    const float *tr = c_near + (size_t)c_tile * kRec32 * kTs + r * kT + tid;
-                    const float tx = (__ldg(tr) - cs.x) + __ldg(tr + 3 * kTs);
-                    const float ty = (__ldg(tr + kTs) - cs.y) + __ldg(tr + 4 * kTs);
-                    const float tz = (__ldg(tr + 2 * kTs) - cs.z) + __ldg(tr + 5 * kTs);
-                    m2x[r] = pack2(-2.0f * tx, -2.0f * tx);
-                    m2y[r] = pack2(-2.0f * ty, -2.0f * ty);
-                    m2z[r] = pack2(-2.0f * tz, -2.0f * tz);
-                    const float b1 = fmaf(tx, tx, fmaf(ty, ty, tz * tz));
-                    bb[r] = pack2(b1, b1);
-                    ax[r] = ay[r] = az[r] = gxs[r] = gys[r] = gzs[r] = 0ull;
-                }
-                const u64 *s2 = reinterpret_cast<const u64 *>(s);  // row k, sources (2m, 2m+1)
-#pragma unroll kFarUnroll
-                for (int m = 0; m < kTs / 2; ++m) {
-                    const u64 sx = s2[m], sy = s2[kTs / 2 + m], sz = s2[kTs + m], sa = s2[3 * (kTs / 2) + m];
-                    const u64 gx = s2[2 * kTs + m], gy = s2[5 * (kTs / 2) + m], gz = s2[3 * kTs + m];
-                    const u64 mx = s2[7 * (kTs / 2) + m], my = s2[4 * kTs + m], mz = s2[9 * (kTs / 2) + m];
-#pragma unroll
-                    for (int r = 0; r < kR; ++r) {
-                        const u64 q = ffma2(sx, m2x[r], ffma2(sy, m2y[r], ffma2(sz, m2z[r], fadd2(sa, bb[r]))));
-                        const u64 iq = rsqrt2(q);
-                        const u64 kk = fmul2(fmul2(iq, iq), iq);
-                        ax[r] = ffma2(kk, mx, ax[r]);
-                        ay[r] = ffma2(kk, my, ay[r]);
-                        az[r] = ffma2(kk, mz, az[r]);
-                        gxs[r] = ffma2(kk, gx, gxs[r]);
-                        gys[r] = ffma2(kk, gy, gys[r]);
-                        gzs[r] = ffma2(kk, gz, gzs[r]);
-                    }
-                }
-#pragma unroll
-                for (int r = 0; r < kR; ++r) {
-                    // t = -m2 / 2 exactly (both lanes of m2 hold -2 t)
-                    const float tx = -0.25f * sum2(m2x[r]), ty = -0.25f * sum2(m2y[r]), tz = -0.25f * sum2(m2z[r]);
-                    const float bx = sum2(gxs[r]), by = sum2(gys[r]), bz = sum2(gzs[r]);
-                    const float vx = sum2(ax[r]) - fmaf(ty, bz, -tz * by);
-                    const float vy = sum2(ay[r]) - fmaf(tz, bx, -tx * bz);
-                    const float vz = sum2(az[r]) - fmaf(tx, by, -ty * bx);
-                    acc[0][r][tid] += __float2ll_rn(vx * c_mult);
-                    acc[1][r][tid] += __float2ll_rn(vy * c_mult);
-                    acc[2][r][tid] += __float2ll_rn(vz * c_mult);
-                }
+                far_tile<false>(s, insts[c_inst].tinfo[un.src], c_near + (size_t)c_tile * kRec32 * kTs + tid, nullptr,
+                                0.0f, 0.0f, c_mult, acc, tid);
+            } else if (kCut && un.far == 3) {
+                far_tile<true>(s, insts[c_inst].tinfo[un.src], c_near + (size_t)c_tile * kRec32 * kTs + tid,
+                               c_near + (size_t)un.src * kRec32 * kTs, c_d2 + c_c2, c_c2, c_mult, acc, tid);
             } else if (!kCut || un.far == 0) {
                 near_tile<false, kR, kT>(s, c_near + (size_t)c_tile * kRec32 * kTs + tid, c_d2, 0.0f, c_mult, acc, tid);
             } else {
