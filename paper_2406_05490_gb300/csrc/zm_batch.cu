@@ -67,11 +67,12 @@ __global__ void __launch_bounds__(kPtb)
     const Inst &I = insts[block_inst[blockIdx.x]];
     const int p = (blockIdx.x - I.block0) * kPtb + threadIdx.x;
     if (p >= I.geom.N || !ZM_IDX_OK(p, I.geom.N)) return;
+    const double ga = -2.0 * I.atwood * I.geom.i12a, gb = -2.0 * I.atwood * I.geom.i12b;
     if (I.mu != 0.0)
-        vorticity_point<true, kMode>(I.geom, p, I.phi, I.y[yin], I.u, I.atwood, I.mu, I.dt, ca, cb,
+        vorticity_point<true, kMode>(I.geom, p, I.phi, I.y[yin], I.u, ga, gb, I.mu, I.dt, ca, cb,
                                      I.y[0], I.y[yout], I.y[2]);
     else
-        vorticity_point<false, kMode>(I.geom, p, I.phi, I.y[yin], I.u, I.atwood, I.mu, I.dt, ca, cb,
+        vorticity_point<false, kMode>(I.geom, p, I.phi, I.y[yin], I.u, ga, gb, I.mu, I.dt, ca, cb,
                                       I.y[0], I.y[yout], I.y[2]);
 }
 

@@ -30,6 +30,7 @@ struct Geom {
     int periodic;
     double i12a, i12b;    // 1 / (12 dx1), 1 / (12 dx2): first-difference weights
     double i12a2, i12b2;  // 1 / (12 dx1^2), 1 / (12 dx2^2): second-difference weights
+    double c8det;         // (144 dx1 dx2)^2 / 8
 };
 
 // Fill in the spacings and stencil weights of a Geom whose n1, n2, L1, L2 are set (on the host,
@@ -43,6 +44,7 @@ inline void geom_finish(Geom &g)
     g.i12b = 1.0 / (12.0 * g.dx2);
     g.i12a2 = 1.0 / (12.0 * g.dx1 * g.dx1);
     g.i12b2 = 1.0 / (12.0 * g.dx2 * g.dx2);
+    g.c8det = (144.0 * g.dx1 * g.dx2) * (144.0 * g.dx1 * g.dx2) / 8.0;
 }
 
 // Source records of the Birkhoff-Rott sum are stored tile-major: a tile is a tp1 x tp2 patch of
@@ -121,6 +123,16 @@ struct Inst {
 };
 
 class Batch;
+
+// Threads per CTA of the kernels with one thread per mesh node: 256, halved (down to a warp) while there
+// would be fewer than two CTAs per SM, so that a small mesh's FP64 work spreads over the SMs (32 x 32
+// nodes: 4 CTAs on 4 SMs -> 32; ten FP64 steps 1799 -> 1695 us).
+inline int point_threads(int N)
+{
+    int t = 256;
+    while (t > 32 && N < 304 * t) t >>= 1;
+    return t;
+}
 
 }  // namespace zm
 
@@ -240,6 +252,9 @@ int df_vorticity(zm_ctx *c, const double *y, double *wdot_out, const double *y0,
 // count values src -> dst, FP64 -> double word (to_df) or back; `state`: src/dst hold the 5N
 // state and z1, z2 are taken relative to the mesh coordinates.  src may equal dst.
 int df_convert(zm_ctx *c, const double *src, double *dst, size_t count, int state, int to_df);
+// The 5N state between FP64 device arrays (z 3N, w 2N; state_out: either may be null) and double words.
+int df_state_in(zm_ctx *c, const double *z, const double *w, double *dst);
+int df_state_out(zm_ctx *c, const double *src, double *z, double *w);
 int df_check_finite(zm_ctx *c, const double *y, size_t nvalues, int *dev_flag);
 
 // ---- one full derivative evaluation (zm_api.cu) --------------------------------------------------
@@ -427,16 +442,15 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return false;
 }
 
-// 1 / sqrt(x) for a positive double inside the FP32 range: the FP32 estimate refined by two
-// Newton-Raphson steps y <- y (3/2 - x/2 y^2) (relative error ~2^-22 -> ~2^-43 -> FP64 rounding),
-// a few FP64 instructions instead of a correctly rounded square root and division.
-__device__ __forceinline__ double rsqrt_nr(double x)
+// 1 / sqrt(x) for a positive, normal double: the hardware estimate (see rsqrt_cube) corrected to second
+// order, y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2; the dropped 5 e^3/16 is below 2^-58.  Five FP64
+// instructions and one MUFU operation.
+__device__ __forceinline__ double rsqrt_f64(double x)
 {
-    const double hx = 0.5 * x;
-    double y = (double)rsqrtf((float)x);
-    y = y * fma(-hx * y, y, 1.5);
-    y = y * fma(-hx * y, y, 1.5);
-    return y;
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 
 // q^(-3/2) for a positive, normal double q: the hardware estimate y ~ q^(-1/2) (PTX

@@ -8,6 +8,9 @@
 //     (Sec. 3.1 TimeIntegrator, three derivative evaluations per step).
 // One thread per mesh node; neighbours come through L1/L2, so each kernel streams its fields
 // once from HBM.
+#include <algorithm>
+#include <cmath>
+
 #include "zm_stencil.cuh"
 
 namespace zm {
@@ -76,12 +79,12 @@ __global__ void __launch_bounds__(kTpb)
 template <bool kVisc, int kMode>
 __global__ void __launch_bounds__(kTpb)
     vorticity_kernel(Geom g, const double *__restrict__ phi, const double *__restrict__ y,
-                     const double *__restrict__ u, double atwood, double mu, double dt, double ca,
+                     const double *__restrict__ u, double ga, double gb, double mu, double dt, double ca,
                      double cb, const double *y0, double *yout, double *__restrict__ wdot)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= g.N) return;
-    vorticity_point<kVisc, kMode>(g, p, phi, y, u, atwood, mu, dt, ca, cb, y0, yout, wdot);
+    vorticity_point<kVisc, kMode>(g, p, phi, y, u, ga, gb, mu, dt, ca, cb, y0, yout, wdot);
 }
 
 __global__ void finite_kernel(size_t n, const double *__restrict__ y, int *bad)
@@ -112,12 +115,18 @@ int launch_geometry(zm_ctx *c, const double *y)
         return set_error(ZM_ERR_INVALID, "geometry pass: missing buffer");
     const Geom &g = c->geom;
     const double pref = g.dx1 * g.dx2 / (4.0 * 3.14159265358979323846);
-    dim3 grid((g.N + kTpb - 1) / kTpb);
+    const int tpb = point_threads(g.N);
+    dim3 grid((g.N + tpb - 1) / tpb);
     cudaEvent_t ev = nullptr;
     prof_begin(c, ZM_K_GEOMETRY, &ev);
-    if (c->order != ZM_ORDER_HIGH)
-        geometry_kernel<kGeoLow><<<grid, kTpb, 0, c->stream>>>(g, c->tiling, y, pref, c->g, nullptr,
-                                                             c->q, c->nrm);
+    if (c->order != ZM_ORDER_HIGH) {
+        const int e1 = std::ilogb(g.L1), e2 = std::ilogb(g.L2);
+        if (std::max(e1, e2) < 100 && std::min(e1, e2) > -100)
+            geometry_kernel<kGeoLow><<<grid, tpb, 0, c->stream>>>(g, c->tiling, y, pref, c->g, nullptr, c->q, c->nrm);
+        else
+            geometry_kernel<kGeoLowWide><<<grid, tpb, 0, c->stream>>>(g, c->tiling, y, pref, c->g, nullptr, c->q,
+                                                                       c->nrm);
+    }
     // FP64 source records (high and medium order); FP32C contexts build theirs in the batch
     if (c->order != ZM_ORDER_LOW && !c->batch) {
         if (c->order == ZM_ORDER_MEDIUM) {  // the second geometry pass of a medium-order evaluation
@@ -128,7 +137,7 @@ int launch_geometry(zm_ctx *c, const double *y)
             const int rc = launch_geometry_dw(c, y, pref);
             if (rc) return rc;
         } else
-            geometry_kernel<kGeoFp64><<<grid, kTpb, 0, c->stream>>>(g, c->tiling, y, pref, c->g, c->src,
+            geometry_kernel<kGeoFp64><<<grid, tpb, 0, c->stream>>>(g, c->tiling, y, pref, c->g, c->src,
                                                               c->q, nullptr);
     }
     prof_end(c, ZM_K_GEOMETRY, ev);
@@ -139,14 +148,15 @@ int launch_reduce(zm_ctx *c, bool write_phi)
 {
     if (!c->part || !c->u || !c->phi || !c->q) return set_error(ZM_ERR_INVALID, "reduction: missing buffer");
     const Geom &g = c->geom;
-    dim3 grid((g.N + kTpb - 1) / kTpb);
+    const int tpb = point_threads(g.N);
+    dim3 grid((g.N + tpb - 1) / tpb);
     cudaEvent_t ev = nullptr;
     prof_begin(c, ZM_K_REDUCE, &ev);
     if (c->plan.nsplit >= 4 * kRedG && g.N <= 16 * kTpb * 152)
         reduce_wide_kernel<<<(g.N + kTpb / kRedG - 1) / (kTpb / kRedG), kTpb, 0, c->stream>>>(
             g.N, c->plan.nsplit, c->part, c->q, c->u, c->phi, write_phi ? 1 : 0);
     else
-        reduce_kernel<<<grid, kTpb, 0, c->stream>>>(g.N, c->plan.nsplit, c->part, c->q, c->u, c->phi,
+        reduce_kernel<<<grid, tpb, 0, c->stream>>>(g.N, c->plan.nsplit, c->part, c->q, c->u, c->phi,
                                                     write_phi ? 1 : 0);
     prof_end(c, ZM_K_REDUCE, ev);
     return cuda_check(cudaGetLastError(), "reduce kernel launch");
@@ -158,17 +168,22 @@ int launch_vorticity(zm_ctx *c, const double *y, double *wdot_out, const double 
     if (!y || !c->phi || !c->u || (mode == 0 && !wdot_out) || (mode == 1 && (!y0 || !yout)))
         return set_error(ZM_ERR_INVALID, "vorticity pass: missing buffer");
     const Geom &g = c->geom;
-    dim3 grid((g.N + kTpb - 1) / kTpb);
+    const int tpb = point_threads(g.N);
+    dim3 grid((g.N + tpb - 1) / tpb);
     cudaEvent_t ev = nullptr;
     prof_begin(c, ZM_K_VORT, &ev);
     const bool visc = (c->mu != 0.0);
+    const double ga = -2.0 * c->atwood * g.i12a, gb = -2.0 * c->atwood * g.i12b;
+    if (mode == 1 && ca == 0.0 && cb == 1.0) mode = 2;
 #define ZM_VORT(V, M)                                                                          \
-    vorticity_kernel<V, M><<<grid, kTpb, 0, c->stream>>>(g, c->phi, y, c->u, c->atwood, c->mu, \
-                                                         dt, ca, cb, y0, yout, wdot_out)
+    vorticity_kernel<V, M><<<grid, tpb, 0, c->stream>>>(g, c->phi, y, c->u, ga, gb, c->mu, dt, ca, cb, y0, yout, \
+                                                         wdot_out)
     if (mode == 0) {
         if (visc) ZM_VORT(true, 0); else ZM_VORT(false, 0);
-    } else {
+    } else if (mode == 1) {
         if (visc) ZM_VORT(true, 1); else ZM_VORT(false, 1);
+    } else {
+        if (visc) ZM_VORT(true, 2); else ZM_VORT(false, 2);
     }
 #undef ZM_VORT
     prof_end(c, ZM_K_VORT, ev);
