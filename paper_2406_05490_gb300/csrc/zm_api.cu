@@ -145,6 +145,19 @@ static bool is_device_ptr(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Whether the context's kernels can read or write p directly: managed memory or memory of the context's
+// own GPU, aligned to its type.
+static bool kernel_ptr(const zm_ctx *c, const double *p)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == c->device)) &&
+           reinterpret_cast<uintptr_t>(p) % sizeof(double) == 0;
+}
+
 static int copy_in(zm_ctx *c, double *dst, const double *src, size_t count)
 {
     const cudaMemcpyKind k = is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
@@ -367,6 +380,7 @@ int zm_set_state(zm_ctx *c, const double *z, const double *w)
 {
     if (!c || !z || !w) return set_error(ZM_ERR_INVALID, "zm_set_state: null argument");
     const size_t N = c->geom.N;
+    if (c->df64 && kernel_ptr(c, z) && kernel_ptr(c, w)) return df_state_in(c, z, w, c->y0);
     double *dst = c->df64 ? c->yb : c->y0;  // double word: stage FP64 in yb, convert into y0
     int rc = copy_in(c, dst, z, 3 * N);
     if (!rc) rc = copy_in(c, dst + 3 * N, w, 2 * N);
@@ -383,6 +397,7 @@ int zm_get_state(zm_ctx *c, double *z, double *w)
     bool host = false;
     int rc = ZM_OK;
     const double *src = c->y0;
+    if (c->df64 && (!z || kernel_ptr(c, z)) && (!w || kernel_ptr(c, w))) return df_state_out(c, c->y0, z, w);
     if (c->df64) {  // FP64 copy of the state in yb (a stage buffer, free between calls)
         rc = df_convert(c, c->y0, c->yb, 5 * N, 1, 0);
         src = c->yb;
@@ -402,7 +417,10 @@ int zm_velocity(zm_ctx *c, const double *z, const double *w, double *u, double *
     const size_t N = c->geom.N;
     const double *y = c->y0;
     int rc = ZM_OK;
-    if (z) {
+    if (z && c->df64 && kernel_ptr(c, z) && kernel_ptr(c, w)) {
+        rc = df_state_in(c, z, w, c->ya);
+        y = c->ya;
+    } else if (z) {
         double *dst = c->df64 ? c->yb : c->ya;
         rc = copy_in(c, dst, z, 3 * N);
         if (!rc) rc = copy_in(c, dst + 3 * N, w, 2 * N);

@@ -420,6 +420,81 @@ __global__ void from_df_kernel(int n2, size_t N, size_t count, double dx1, doubl
     }
 }
 
+// The state between the caller's FP64 device arrays and double-word storage, one thread per node and no
+// staging copy.  Bound by the FP64 pipe as long as each value took four FP64 conversions and sums to
+// split and three to join (4096 x 4096: 1.9 ms in and out); the words are cut and joined with integer
+// operations instead, and FP64 is left with the mesh coordinate and one sum (0.61 ms in and out).
+
+// The plain conversions, for the values outside the integer forms' range; not inlined, or the compiler
+// runs their FP64 instructions for every value and selects.
+__device__ __noinline__ float2 split_plain(double v)
+{
+    const float hi = __double2float_rn(v);
+    return make_float2(hi, __double2float_rn(v - (double)hi));
+}
+__device__ __noinline__ double widen_plain(float f) { return (double)f; }
+
+// v = hi + lo, hi the nearest FP32 number, lo the rest rounded to FP32.
+__device__ __forceinline__ float2 split_fast(double v)
+{
+    const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
+    const int e = (int)((h >> 20) & 0x7ff);
+    if (e < 1023 - 60 || e > 1023 + 100) return split_plain(v);  // zero, tiny or huge
+    // the leading 24 bits, rounded, and the signed rest of the 53, in units of 2^(e - 1075)
+    const unsigned m = ((h & 0xfffffu) << 3) | (l >> 29);
+    const unsigned up = (l >> 28) & 1u;
+    const unsigned sign = h & 0x80000000u;
+    const float hi = __uint_as_float((((unsigned)(e - 896) << 23) + m + up) | sign);
+    const int rest = (int)(l & 0x1fffffffu) - (int)(up << 29);
+    const float lo = (float)rest * __uint_as_float(((unsigned)(e - 1075 + 127) << 23) | sign);
+    return make_float2(hi, lo);
+}
+
+// A FP32 number as FP64.
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned b = __float_as_uint(f), a = b & 0x7fffffffu;
+    if (a - 0x00800000u >= 0x7f000000u) return widen_plain(f);  // zero, denormal or not finite
+    return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+__global__ void __launch_bounds__(kTpb)
+    state_in_kernel(DfGeo g, double dx1, double dx2, const double *__restrict__ z, const double *__restrict__ w,
+                    float2 *__restrict__ y)
+{
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= g.N || !ZM_IDX_OK(p, g.N)) return;
+    int i, j;
+    node_ij<false>(p, g, i, j);
+    const int N = g.N;
+    y[p] = split_fast(z[p] - __dmul_rn((double)i, dx1));
+    y[N + p] = split_fast(z[N + p] - __dmul_rn((double)j, dx2));
+    y[2 * N + p] = split_fast(z[2 * N + p]);
+    y[3 * N + p] = split_fast(w[p]);
+    y[4 * N + p] = split_fast(w[N + p]);
+}
+
+__global__ void __launch_bounds__(kTpb)
+    state_out_kernel(DfGeo g, double dx1, double dx2, const float2 *__restrict__ y, double *__restrict__ z,
+                     double *__restrict__ w)
+{
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= g.N || !ZM_IDX_OK(p, g.N)) return;
+    int i, j;
+    node_ij<false>(p, g, i, j);
+    const int N = g.N;
+    auto join = [](float2 f) { return widen(f.x) + widen(f.y); };
+    if (z) {
+        z[p] = join(y[p]) + __dmul_rn((double)i, dx1);
+        z[N + p] = join(y[N + p]) + __dmul_rn((double)j, dx2);
+        z[2 * N + p] = join(y[2 * N + p]);
+    }
+    if (w) {
+        w[p] = join(y[3 * N + p]);
+        w[N + p] = join(y[4 * N + p]);
+    }
+}
+
 __global__ void finite_f32_kernel(size_t n, const float *__restrict__ y, int *bad)
 {
     for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n;
@@ -727,6 +802,24 @@ int df_convert(zm_ctx *c, const double *src, double *dst, size_t count, int stat
         to_df_kernel<<<grid, kTpb, 0, c->stream>>>(G.n2, G.N, count, G.dx1, G.dx2, state, src, F2(dst));
     else
         from_df_kernel<<<grid, kTpb, 0, c->stream>>>(G.n2, G.N, count, G.dx1, G.dx2, state, F2(src), dst);
+    return cuda_check(cudaGetLastError(), "double-word conversion launch");
+}
+
+int df_state_in(zm_ctx *c, const double *z, const double *w, double *dst)
+{
+    if (!z || !w || !dst) return set_error(ZM_ERR_INVALID, "double-word conversion: missing buffer");
+    const Geom &G = c->geom;
+    const int tpb = point_threads(G.N);
+    state_in_kernel<<<(G.N + tpb - 1) / tpb, tpb, 0, c->stream>>>(make_geo(c), G.dx1, G.dx2, z, w, F2(dst));
+    return cuda_check(cudaGetLastError(), "double-word conversion launch");
+}
+
+int df_state_out(zm_ctx *c, const double *src, double *z, double *w)
+{
+    if (!src) return set_error(ZM_ERR_INVALID, "double-word conversion: missing buffer");
+    const Geom &G = c->geom;
+    const int tpb = point_threads(G.N);
+    state_out_kernel<<<(G.N + tpb - 1) / tpb, tpb, 0, c->stream>>>(make_geo(c), G.dx1, G.dx2, F2(src), z, w);
     return cuda_check(cudaGetLastError(), "double-word conversion launch");
 }
 
