@@ -473,8 +473,9 @@ def bench_low_order(zm, torch, inputs, flush, nl, steps, warmup, df64, fp64_tflo
             "steps": steps, "steps_per_s": steps / (msl * 1e-3), "ms_per_step": msl / steps,
             "step_alg_gbs": step_bytes / (msl / steps * 1e-3) / 1e9,
             "step_hbm_frac": step_bytes / (msl / steps * 1e-3) / 1e9 / HBM_GBS,
-            "issue_basis": ("ncu-counted warp instructions per point (profiles/df64_issue_instructions.json)"
-                            " x points / time / (SMs x 4 schedulers x sampled SM clock)") if df64 and issue_rate else None,
+            "issue_basis": ("ncu-counted warp instructions per point (profiles/%s_instructions.json)"
+                            " x points / time / (SMs x 4 schedulers x sampled SM clock)"
+                            % ("df64_issue" if df64 else "fp64_pipe")) if issue_rate else None,
             "riesz_floor_gbs": 80 * pts / (kern["fft"]["ms_per_eval"] * 1e-3) / 1e9
             if kern["fft"]["ms_per_eval"] > 0 else 0.0,
             "kernels": kern, "hbm_peak_gbs": HBM_GBS, "hbm_peak_basis": "measured copy bandwidth",
