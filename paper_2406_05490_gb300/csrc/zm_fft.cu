@@ -22,11 +22,11 @@
 // butterflies.  Each CTA leaves the exponent of its unit beside its output, and the largest one
 // in a word that the next pass aligns its input to.  A value that is not finite sets that word
 // beyond every exponent, and all results are NaN, as they would be in FP64.
-// ms per evaluation, FP64 butterflies / integers: 1024^2 0.452 / 0.111, 4096^2 6.85 / 1.44, 4864^2 13.18 /
-// 2.88, 512^2 0.117 / 0.053, 152 x 304 0.138 / 0.064, 128^2 0.031 / 0.033 (latency).  Relative error of u
-// against a long double transform: 256^2 4.7e-16 / 4.4e-16, 512^2 5.6e-16 / 5.2e-16, 152 x 304 5.5e-16 /
-// 5.4e-16.  What bounds it now: latency at 16 warps per SM (128 registers for 16 values), the schedulers
-// issuing in 30 to 45 % of cycles.
+// ms per evaluation, FP64 butterflies / integers: 1024^2 0.452 / 0.102, 4096^2 6.85 / 1.44, 4864^2 13.18 /
+// 2.88, 512^2 0.115 / 0.052, 152 x 304 0.138 / 0.064, 128^2 0.031 / 0.029 (latency).  Relative error of u
+// against a long double transform: 128^2 3.8e-16 / 3.2e-16, 256^2 4.7e-16 / 4.3e-16, 512^2 5.6e-16 /
+// 5.2e-16, 152 x 304 5.5e-16 / 5.3e-16, 608 x 152 5.5e-16 / 5.6e-16.  What bounds it now: latency at 16 warps per SM (128 registers for 16 values), the schedulers
+// issuing in 34 to 47 % of cycles.
 //
 // Sides L = R M with M = 2^a (a >= 3) and R odd (3 .. 19; 4864 = 19 x 256 is the paper's
 // low-order mesh, Sec. 5.1) add one radix-R stage: before the length-M transforms in decimation
@@ -516,12 +516,10 @@ __global__ void __launch_bounds__(threads_for(A, kMix), minb_for(A, kMix))
     mx = words[0];
     // |w| < 2^eb; to integers below 2^54
     const int eb = max((int)(mx >> 20) - 1022, -940);
-    const double sc = __hiloint2double((1023 + 54 - eb) << 20, 0);
     unsigned o = 0;
     for (int e = threadIdx.x; e < rows * L; e += blockDim.x) {  // the thread's own elements
         const ulonglong2 v = sx[phys(e)];
-        const Z a{__double2ll_rn(__longlong_as_double((long long)v.x) * sc),
-                  __double2ll_rn(__longlong_as_double((long long)v.y) * sc)};
+        const Z a{fix_of(v.x, eb), fix_of(v.y, eb)};
         or_mag(o, a);
         sx[phys(e)] = stz(a);
     }
@@ -648,10 +646,9 @@ __global__ void __launch_bounds__(threads_for(A, kMix), minb_for(A, kMix))
         __syncthreads();
         rows_dif<A, kMix>(sx, rows, s2, +1, un, &words[kNorm]);
     }
-    // -s/2 per unit, as two factors (the exponent may lie outside the range of one)
-    const int e1 = data ? un.e / 2 : 0, e2 = data ? un.e - e1 : 0;
-    const double f1 = finite ? -0.5 * inv * __hiloint2double((1023 + e1) << 20, 0) : __longlong_as_double(0x7ff8000000000000ll);
-    const double f2 = __hiloint2double((1023 + e2) << 20, 0);
+    // -s/2 per unit as 2^e1 in the conversion and a factor (the exponent may lie outside the range of one)
+    const int e1 = data ? min(max(un.e, -800), 800) : 0, e2 = data ? un.e - e1 : 0;
+    const double f2 = finite ? -0.5 * inv * __hiloint2double((1023 + e2) << 20, 0) : __longlong_as_double(0x7ff8000000000000ll);
     const int total = rows * L, step = blockDim.x % L, rstep = blockDim.x / L;
     int r = threadIdx.x / L, j = threadIdx.x % L;
     constexpr int kB = kBatch / 2;
@@ -667,7 +664,7 @@ __global__ void __launch_bounds__(threads_for(A, kMix), minb_for(A, kMix))
                 n1v[b] = __ldcs(nrm + N + p);
                 n2v[b] = __ldcs(nrm + 2 * N + p);
                 qv[b] = __ldcs(q + p);
-                s[b] = (double)(data ? ldz(sx[phys(k)]).re : 0ll) * f1 * f2;
+                s[b] = fp64_of(data ? ldz(sx[phys(k)]).re : 0ll, e1) * f2;
             }
             r += rstep;
             j += step;
