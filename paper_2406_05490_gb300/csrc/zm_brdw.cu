@@ -481,8 +481,12 @@ __global__ void __launch_bounds__(kTs, 7) brdw_kernel(const DwArgs a)
             if ((mask >> k) & 1) dev::tma_load_1d(stage[b], a.far_rec + s * kFarWords, kFarBytes, &bar[b]);
             else dev::tma_load_1d(stage[b], a.near_rec + s * kNearWords, kNearBytes, &bar[b]);
         };
-        if (tid == 0)
+        if (tid == 0) {
+            // both stages were read by the last 64 tiles: order those reads (ended by the barrier
+            // above) before the copies that overwrite them
+            dev::fence_proxy_async();
             for (int k = 0; k < 2 && k < n; ++k) issue(k, (unit + k) & 1);
+        }
         for (int k = 0; k < n; ++k, ++unit) {
             const int b = unit & 1;
             const bool ok = dev::mbar_wait_bounded(&bar[b], (unit >> 1) & 1);
