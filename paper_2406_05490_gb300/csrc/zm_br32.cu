@@ -70,16 +70,17 @@ struct Unit {
 
 // Far pair terms of one source tile (stage `s`) for this thread's kR targets (near-record row pointer
 // tr0, kT apart); cs: the source tile's centre.
-// kMask: the tile pair straddles the cutoff; only pairs with |r|^2 <= c2 count, thr = c2 + delta^2.  The
-// Gram form decides, except for pairs closer to the cutoff than its own error, which is below
+// kMask: the tile pair straddles the cutoff; only pairs with |r|^2 <= c2 count, thr = c2 + d2, d2 =
+// delta^2.  The Gram form decides, except for pairs closer to the cutoff than its own error, which is below
 // 11 2^-24 (|s| + |t|)^2 (the roundings of s, t, their squares and the four sums) <= 2^-19 (|t|^2 +
-// radius^2); about one pair in 10^5 is as close.  Those are decided as near_tile does, on the FP32
-// hi/lo difference (source record src_near), and their q is moved to their side of thr.  (The near
-// form for all of these pairs, 23 FP32 operations and the mask against 12 and the mask: 512 x 512,
-// cutoff 0.2: 9.9 against 7.3 ms per evaluation.)
+// radius^2), and 8 2^-24 d2, since d2 takes part in the three sums of |s|^2 + d2, the four after them and
+// thr; with a core of a fraction of the cutoff about one pair in 10^5 is as close.  Those are decided as
+// near_tile does, on the FP32 hi/lo difference (source record src_near), and their q is moved to their
+// side of thr.  (The near form for all of these pairs, 23 FP32 operations and the mask against 12 and the
+// mask: 512 x 512, cutoff 0.2: 9.9 against 7.3 ms per evaluation.)
 template <bool kMask>
 __device__ __forceinline__ void far_tile(const float *s, const float4 cs, const float *__restrict__ tr0,
-                                         const float *__restrict__ src_near, float thr, float c2, float mult,
+                                         const float *__restrict__ src_near, float d2, float c2, float mult,
                                          long long (*acc)[kR][kT], int tid)
 {
     u64 m2x[kR], m2y[kR], m2z[kR], bb[kR];
@@ -99,8 +100,10 @@ __device__ __forceinline__ void far_tile(const float *s, const float4 cs, const 
         if (kMask) bmax = r ? fmaxf(bmax, b1) : b1;
         ax[r] = ay[r] = az[r] = gxs[r] = gys[r] = gzs[r] = 0ull;
     }
+    const float thr = d2 + c2;
     const u64 nthr = pack2(-thr, -thr);
-    const float eps = (bmax + cs.w * cs.w) * 1.9073486328125e-6f;  // 2^-19 (|t|^2 + radius^2)
+    // 2^-19 (|t|^2 + radius^2) + 2^-20 d2
+    const float eps = (bmax + cs.w * cs.w) * 1.9073486328125e-6f + d2 * 9.5367431640625e-7f;
     const u64 *s2 = reinterpret_cast<const u64 *>(s);  // row k, sources (2m, 2m+1)
 #pragma unroll kFarUnroll
     for (int m = 0; m < kTs / 2; ++m) {
@@ -175,8 +178,8 @@ __device__ __forceinline__ void far_tile(const float *s, const float4 cs, const 
     }
 }
 
-// kCut: some interface of the batch sums within a cutoff, so straddling tile pairs (masked
-// near path) can occur; without it that path is compiled out.
+// kCut: some interface of the batch sums within a cutoff, so straddling tile pairs (the masked
+// forms of both paths) can occur; without it those are compiled out.
 template <bool kCut>
 __global__ void __launch_bounds__(kT, ZM_BR32_MINB)
     br32_batch_kernel(const Inst *__restrict__ insts, int ninst, long long nitems,
@@ -320,7 +323,7 @@ __global__ void __launch_bounds__(kT, ZM_BR32_MINB)
                                 0.0f, 0.0f, c_mult, acc, tid);
             } else if (kCut && un.far == 3) {
                 far_tile<true>(s, insts[c_inst].tinfo[un.src], c_near + (size_t)c_tile * kRec32 * kTs + tid,
-                               c_near + (size_t)un.src * kRec32 * kTs, c_d2 + c_c2, c_c2, c_mult, acc, tid);
+                               c_near + (size_t)un.src * kRec32 * kTs, c_d2, c_c2, c_mult, acc, tid);
             } else if (!kCut || un.far == 0) {
                 near_tile<false, kR, kT>(s, c_near + (size_t)c_tile * kRec32 * kTs + tid, c_d2, 0.0f, c_mult, acc, tid);
             } else {
