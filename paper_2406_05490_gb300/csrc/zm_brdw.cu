@@ -3,85 +3,79 @@
 // rounding decides the result:
 //     u_i = sum_j (z_j - z_i) x gamma'_j / (|z_j - z_i|^2 + delta^2)^(3/2).
 //
-// What bounds it.  GB300 executes 2 FP64 instructions per clock and SM against 128 FP32 ones, so
-// the 21 FP64 instructions of a pair (zm_br.cu) cost 10.5 clocks of an SM whose other pipes idle
-// (measured: the pipe 90 % busy, 190 ms per 256 x 256 evaluation).  A pair far apart compared with
-// its source tile is evaluated here in FP32 pairs and integers instead: 53 FP32 lane
-// operations (two lanes per packed instruction), 6 integer multiply-adds 32 x 32 + 64 bits, one
-// reciprocal square root and one conversion, about half a clock of the FMA pipe, which bounds it.
-// 190.3 -> 12.5 ms at 256 x 256, 13.0 -> 1.2 at 128 x 128, 7.5 -> 0.70 at 90 x 131, 0.81 -> 0.27 at
-// 64 x 64 (one evaluation).
+// What bounds it.  GB300 executes 2 FP64 instructions per clock and SM, so the 21 FP64 instructions of
+// a pair (zm_br.cu) cost 10.5 clocks of an SM whose other pipes idle (measured: the pipe 90 % busy, 190 ms
+// per 256 x 256 evaluation).  A pair far apart compared with its source tile is evaluated here in 64-bit
+// integers instead, to the same precision: 29 integer multiply-adds 32 x 32 + 64 bits (about 30 per clock
+// and SM), some 50 other integer operations, 9 in FP32, one reciprocal square root: 1.5 clocks, the multiply
+// and ALU pipes 53 and 51 % busy, together what the schedulers dispatch.
+// 190.3 -> 21.4 ms at 256 x 256, 13.0 -> 1.63 at 128 x 128, 7.5 -> 0.93 at 90 x 131, 0.81 -> 0.23 at
+// 64 x 64 (one evaluation).  (q and K as FP32 pairs take 12.5 ms at 256 x 256 but hold a far pair to 2^-46
+// only: u is then 2e-14 off, relative, where all strength lies further away than the near tiles.)
 //
 // Tiles.  8 x 8 mesh patches (64 nodes) serve as target tiles (one CTA of 64 threads, one target
 // per thread) and as source tiles, staged by 1D bulk TMA.  Small tiles keep the near region, whose
-// pairs cost 20 times as much, small; where a source tile is not far from the target tile, its
-// four quarters (4 x 4 nodes) are classified against each warp's 32 targets.  Measured at 256 x
-// 256 / 128 x 128: without the quarters 17.4 / 1.94 ms, with them 15.6 / 1.27.  By bounding spheres:
+// pairs cost 7 times as much, small; where a source tile is not far from the target tile, its
+// four quarters (4 x 4 nodes) are classified against each warp's 32 targets.  By bounding spheres:
 //   far   (centres at least kappa source radii plus the targets' radius apart): the form below;
 //   near  FP64 throughout, as in zm_br.cu, on the untouched positions and strengths.
 // A tile's near neighbours spread over the source splits (the splits take the tiles in turn).
-// Near pairs carry most of the sum's rounding error: a sheet's pair terms fall off as 1/r^2,
-// so the root sum square of all terms beyond R is 0.14 dx / R of the strength, and an independent
-// relative error of 1e-14 in them is lost in the FP64 rounding of the near terms and of the sum
-// itself.  What a target and a source tile have in common (t, |t|^2, the final products) is kept
-// in FP64 or exact, since its error would not average out over the tile.
 //
-// Far pairs.  Everything is relative to the source tile's centre c: s_j = z_j - c, t_i = z_i - c
-// (exact differences of fixed-point words, below), |s| <= |t| / 2, and
-//   q = (|t|^2 + delta^2) + |s|^2 - 2 s . t   as an FP32 pair: a power of two C above the first term is
-//       added to the running sum, so that no partial sum falls below half of the one before it, the
-//       difference of two of them is exact and one FMA returns the rounding error of the product added;
-//   K = q^(-3/2) from the special-function estimate y: e = 1 - q y^2 with y^2 exact,
-//       y^3 (1 + 3e/2 + 15e^2/8), as FP32 pair (kh, kl);
-//   sums G = sum K g, M = sum K (s x g), and u_tile = M - t x G.  K's leading part is
-//       scaled to an integer below 2^30 (in a far tile K varies by less than 27, so all of its
-//       24 bits are integer bits), g to 27 bits, and K g accumulates exactly in 64-bit integers;
-//       the remainders' products, 2^-26 of the terms, accumulate in FP32.  (FP32-pair sums lost
-//       up to 2e-14: their low words grow with the number of terms.)
-// Positions enter as three words on grids 2^-20, 2^-44 and below (scaled by the mesh's length), so
-// that t = z - c has exact word differences.  Tiles whose coordinates, radius or strength do not
-// fit these ranges (or are not finite) have an infinite radius, that is, are near to all.
+// Far pairs.  Everything is relative to the source tile's centre c: s_j = z_j - c, t_i = z_i - c, FP64
+// differences, so that the origin of the coordinates does not matter.  Per target and tile, in units 2^m in
+// which the least q of the tile has 58 bits:
+//   q = (|t|^2 + delta^2) + |s|^2 - 2 s . t   in 64 bits, the products of the leading 31-bit limbs exact, those
+//       of the remainders, 2^-30 of them, in FP32;
+//   K = q^(-3/2) from the special-function estimate Y of q^(-1/2), taken as an integer: e = 1 - q Y^2 to
+//       2^-52 from the products of the 32-bit limbs, K = Y^3 (1 + 3/2 e + 15/8 e^2) to 2^-57 (the square in FP32);
+//   sums G = sum K g, M = sum K (s x g), and u_tile = M - t x G.  K has a leading limb below 2^30 and a
+//       trailing one of 28 bits (in a far tile K varies by less than 26), g 26 and 28 bits; the products of the
+//       leading limbs and the mixed ones accumulate exactly in 64-bit integers.
+// Shifts that round down have the mean of what they drop made up for by a constant, since the error of
+// a tile's pairs would not average out.  Tiles whose radius or strength does not fit (or is not finite) have an
+// infinite radius, that is, are near to all.
 //
-// Accuracy of u against long double sums (multi-mode interface, relative L2 over sampled targets;
-// zm_br.cu's plain FP64 sum / here): 56 x 56 7.5e-16 / 5.1e-16, 80 x 80 4.7e-16 / 5.6e-16, 96 x 96
-// 8.2e-16 / 6.3e-16, 90 x 131 1.2e-15 / 7.5e-16, 128 x 128 1.5e-15 / 7.1e-16, 256 x 256 5.7e-15 /
-// 6.9e-16: the long FP64 sums rounded more than the far pairs lose.
+// Accuracy.  One source node's contribution, relative, rms over random positions: 2.3e-16 (4.5e-16 at the
+// edge of the far region; the FP64 pair 1.5e-16); 64 random strengths in a tile 3.7e-16 (5.1e-16), 64 alike
+// 1.2e-16 (2.2e-16).  u against long double sums (multi-mode interface, relative L2 over sampled
+// targets; zm_br.cu's plain FP64 sum / here): 56 x 56 7.5e-16 / 2.0e-16, 80 x 80 4.7e-16 / 2.6e-16, 96 x 96
+// 8.2e-16 / 2.8e-16, 90 x 131 1.2e-15 / 2.4e-16, 128 x 128 1.5e-15 / 2.6e-16, 200 x 150 1.8e-15 / 2.7e-16,
+// 256 x 256 5.7e-15 / 5.1e-16: the plain sums are longer.
 #include <algorithm>
 #include <cmath>
 
-#include "zm_df64.cuh"
+#include "zm_fix.cuh"
 #include "zm_stencil.cuh"
 
 namespace zm {
 namespace {
 
-using namespace dw;
-
 constexpr int kT = 8;         // tile side
 constexpr int kTs = kT * kT;  // nodes per tile, threads per CTA
 constexpr int kSub = 4;       // a tile's quarters: 4 x 4 nodes
 constexpr int kNearRows = 6;  // FP64: position, scaled strength
-// far rows (32-bit words): s hi (3), s lo (3), |s|^2 hi, lo, g and s x g as integers (6), their
-// remainders (6), both as FP32 (6)
-constexpr int kFarRows = 26;
-constexpr int kRowA = 6, kRowI = 8, kRowR = 14, kRowF = 20;
-constexpr int kFarWords = kFarRows * kTs;  // the far record of a tile, or of its four quarters
-// the near block of a tile: its quarters' far records (quarter k in columns 16 k ..) and the FP64 record
+// Far record of a node, 24 words side by side: s as integers (3), as FP32 (3) and the integers' remainders
+// (3), |s|^2 (2), leading (6) and trailing (6) limbs of g and s x g, one word of padding.
+constexpr int kNodeWords = 24;
+constexpr int kFarWords = kNodeWords * kTs;  // the far record of a tile, or of its four quarters
+// the near block of a tile: its quarters' far records (quarter k from node 16 k on) and the FP64 record
 constexpr int kNearWords = kFarWords + 2 * kNearRows * kTs;
-constexpr int kGBits = 26;  // g and s x g: integers below 2^26 in magnitude
-constexpr double kGrid1 = 1048576.0, kGrid2 = 17592186044416.0;  // 2^20, 2^44
+constexpr int kGBits = 26, kGLow = 28;  // g and s x g: n 2^-26 + l 2^-54, |l| <= 2^27
 
 constexpr float kInf = __builtin_huge_valf();
+constexpr float kMaxLength = 1048576.0f;  // 2^20: distances and radii of far tiles, scaled
+
+// Classification: 2 source radii, and a sixteenth so that the bounds of far_tile's integers hold with
+// the rounding of the radii (3 radii: 27.7 against 27.0 ms at 256 x 256 with an earlier form, 2.10 against 1.96
+// at 128 x 128).
+constexpr float kKappa = 2.0625f;
 
 // One tile as the pair kernel sees it.
 struct __align__(16) DwTile {
-    float c1[3], c2[3], c3[3];  // centre, scaled, as fixed-point words
-    float rho;                  // radius, scaled (infinite: near to all)
-    int es;                     // |s| <= rho < 2^es
-    float pad;
-    double gs;                  // 2^(strength exponent) x 2^(-2 length exponent)
-    double c[3];                // centre, scaled
-    double pad2[2];
+    double c[3];   // centre, scaled
+    double gs[2];  // 2^(strength exponent) x 2^(-2 length exponent); the same times sqrt 2
+    float rho;     // radius, scaled (infinite: near to all)
+    int es;        // |s| <= rho < 2^es
 };
 
 // A tile and its quarters.
@@ -126,72 +120,173 @@ __device__ __forceinline__ Patch quarter_of(const Patch &p, int k)
     return q;
 }
 
-// a = w1 + w2 + w3 exactly up to 2^-69: multiples of 2^-20 and 2^-44, and the rest.
-__device__ __forceinline__ void words3(double a, float &w1, float &w2, float &w3)
-{
-    const double g1 = rint(a * kGrid1) * (1.0 / kGrid1);
-    const double r1 = a - g1;
-    const double g2 = rint(r1 * kGrid2) * (1.0 / kGrid2);
-    w1 = __double2float_rn(g1);
-    w2 = __double2float_rn(g2);
-    w3 = __double2float_rn(r1 - g2);
-}
-
 __device__ __forceinline__ unsigned hi_abs(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 
 // Exponent e with rho < 2^e <= 2 rho.
 __device__ __forceinline__ int exp_above(float rho) { return (int)(__float_as_uint(rho) >> 23) - 126; }
 __device__ __forceinline__ double pow2d(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
-// Writes one node's far-record column: s = position relative to the centre (|s| < 2^es), gg =
-// strength below 1; s x g in units of 2^es.
+// ---- the far form --------------------------------------------------------------------------------------
+
+// c + a b; unsigned factors
+__device__ __forceinline__ unsigned long long mad_wu(unsigned a, unsigned b, unsigned long long c)
+{
+    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
+    return c;
+}
+__device__ __forceinline__ unsigned hi32(unsigned long long v) { return (unsigned)(v >> 32); }
+
+// round(v 2^b), |v 2^b| < 2^61, from the bits of v (no FP64 instructions); ties away from zero.
+__device__ __forceinline__ long long fixed(double v, int b)
+{
+    const int hi = __double2hiint(v);
+    const unsigned long long m = ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(v))
+                                 << 8;
+    const int n = min(1083 - ((hi >> 20) & 0x7ff) - b, 63);  // v = m 2^(e - 1083)
+    const long long r = (long long)((m + ((1ull << n) >> 1)) >> n);
+    return hi < 0 ? -r : r;
+}
+// |v| as FP32, truncated (0 below 2^-126); |v| < 2^127.
+__device__ __forceinline__ float abs_f32(double v)
+{
+    const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
+    return h < (897u << 20) ? 0.0f
+                            : __uint_as_float(((h << 3) | ((unsigned)__double2loint(v) >> 29)) - (896u << 23));
+}
+
+// Writes one node's far record: s = position relative to the centre (|s| < 2^es), gg = strength
+// below 1; s x g in units of 2^es.
 __device__ __forceinline__ void put_far(float *__restrict__ fr, const double s[3], const double gg[3], int es)
 {
     const double iu = pow2d(-es);
     const double t[3] = {s[0] * iu, s[1] * iu, s[2] * iu};
     const double g6[6] = {gg[0], gg[1], gg[2], t[1] * gg[2] - t[2] * gg[1], t[2] * gg[0] - t[0] * gg[2],
                           t[0] * gg[1] - t[1] * gg[0]};
+    int *w = reinterpret_cast<int *>(fr);
     double a2 = 0.0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        a2 = fma(s[k], s[k], a2);
-        const float sh = __double2float_rn(s[k]);
-        fr[k * kTs] = sh;
-        fr[(3 + k) * kTs] = __double2float_rn(s[k] - (double)sh);
+        a2 = fma(t[k], t[k], a2);
+        const double v = t[k] * 1073741824.0, n = rint(v);  // 2^30
+        w[k] = __double2int_rn(n);
+        fr[3 + k] = __double2float_rn(v);
+        fr[6 + k] = __double2float_rn(v - n);
     }
-    const float ah = __double2float_rn(a2);
-    fr[kRowA * kTs] = ah;
-    fr[(kRowA + 1) * kTs] = __double2float_rn(a2 - (double)ah);
+    const long long A = __double2ll_rn(a2 * 4611686018427387904.0);  // 2^62
+    w[9] = (int)(unsigned)A;
+    w[10] = (int)(A >> 32);
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-        const double n = rint(g6[k] * (1 << kGBits));
-        fr[(kRowI + k) * kTs] = __int_as_float(__double2int_rn(n));
-        fr[(kRowR + k) * kTs] = __double2float_rn(g6[k] - n * (1.0 / (1 << kGBits)));
-        fr[(kRowF + k) * kTs] = __double2float_rn(g6[k]);
+        const double v = g6[k] * (double)(1 << kGBits), n = rint(v);
+        w[11 + k] = __double2int_rn(n);
+        w[17 + k] = __double2int_rn((v - n) * (double)(1 << kGLow));
     }
 }
+
+// The far pairs of one target and one source tile (records of `count` nodes in shared memory): adds
+// sum_j K (s - t) x g to u.  td: the target, scaled; d2: delta^2, scaled.
+__device__ __forceinline__ void far_tile(const float *__restrict__ rec, int count, const double td[3],
+                                         const DwTile &T, double d2, float d2f, double u[3])
+{
+    const double e[3] = {td[0] - T.c[0], td[1] - T.c[1], td[2] - T.c[2]};
+    // the unit 2^m of q: its least value in the tile, (|t| - rho)^2 + delta^2, lies in [2^57, 2^58)
+    const float fx = abs_f32(e[0]), fy = abs_f32(e[1]), fz = abs_f32(e[2]);
+    const float t2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+    const float tm = fmaf(t2, dev::rsqrt_approx(t2), -T.rho);
+    const int m = (int)(__float_as_uint(fmaf(tm, tm, d2f) * 0.9999f) >> 23) - (127 + 57);
+    // t in units 2^-b with 2 b + m = 62 - odd, and its square in units of q, from limbs of 31 bits
+    const int b = (62 - m) >> 1, odd = m & 1;
+    long long t[3], hi = 0, mid = 0, lo = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        t[k] = fixed(e[k], b);
+        const int h = (int)((t[k] + (1 << 30)) >> 31), l = (int)(t[k] - ((long long)h << 31));
+        hi = mad_w(h, h, hi);
+        mid = mad_w(h, l, mid);
+        lo = mad_w(l, l, lo);
+    }
+    const long long B = (hi << odd) + ((mid + (lo >> 32) + (1 << (29 - odd))) >> (30 - odd)) + fixed(d2, -m);
+    // -2 t in units 2^(m - es + 30), whose products with s (units 2^(es - 30)) are in units of q
+    const int rt = min(b + m - T.es - 1, 63), ra = min(m - 2 * T.es + 62, 63);
+    const long long half = (long long)((1ull << rt) >> 1);
+    int th[3];
+    float tf[3], tl[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const long long v = -((t[k] + half) >> rt);
+        th[k] = (int)((v + (1 << 29)) >> 30);
+        tf[k] = (float)th[k];
+        tl[k] = (float)(int)(v - ((long long)th[k] << 30)) * 9.313225746154785e-10f;  // 2^-30
+    }
+
+    long long I[6] = {0, 0, 0, 0, 0, 0}, J[6] = {0, 0, 0, 0, 0, 0};
+    const int4 *r = reinterpret_cast<const int4 *>(rec);
+#pragma unroll 2
+    for (int j = 0; j < count; ++j, r += kNodeWords / 4) {
+        const int4 w0 = r[0], w1 = r[1], w2 = r[2], w3 = r[3], w4 = r[4], w5 = r[5];
+        // q = |t|^2 + delta^2 - 2 t . s + |s|^2: the remainders' products, 2^-30 of the terms, in FP32
+        const long long h = mad_w(w0.z, th[2], mad_w(w0.y, th[1], mad_w(w0.x, th[0], B)));
+        const float s0 = __int_as_float(w0.w), s1 = __int_as_float(w1.x), s2 = __int_as_float(w1.y);
+        const float l0 = __int_as_float(w1.z), l1 = __int_as_float(w1.w), l2 = __int_as_float(w2.x);
+        float c = fmaf(s2, tl[2], fmaf(s1, tl[1], s0 * tl[0]));
+        c = fmaf(l2, tf[2], fmaf(l1, tf[1], fmaf(l0, tf[0], c)));
+        const long long a = (long long)((unsigned long long)(unsigned)w2.z << 32 | (unsigned)w2.y);
+        const unsigned long long q = (unsigned long long)(h + __float2int_rn(c) + (a >> ra));
+        // Y = 2^60 q^(-1/2) (1 - e/2 ..) and W = Y^2; e = 1 - q W 2^-120, in units 2^-56, then 2^-52 (8: to
+        // round; -1: the mean of what the limbs' products drop)
+        const unsigned qh = hi32(q), ql = (unsigned)q;
+        const unsigned Y = __float2uint_rn(dev::rsqrt_approx(__uint2float_rn(qh)) * 17592186044416.0f);  // 2^44
+        const unsigned long long W = mad_wu(Y, Y, 0);
+        const unsigned wh = hi32(W), wl = (unsigned)W;
+        const unsigned long long x = mad_wu(ql, wh, mad_wu(qh, wl, 0));
+        const int e1 = (int)(((long long)((1ull << 56) + 8 - 1 - mad_wu(qh, wh, 0)) - hi32(x)) >> 4);
+        // e + 1.25 e^2, the square in FP32, as integer by the constant 1.5 2^23
+        const float ef = __int2float_rn(e1);
+        const int ec = e1 + (int)(__float_as_uint(fmaf(ef * 2.7755575615628914e-16f, ef, 12582912.0f)) - 0x4b400000u);
+        // K = Y^3 2^-33 (1 + 3/2 (e + 1.25 e^2)) = 2^147 q^(-3/2) (Y is even, having 24 leading bits; 9: the means of
+        // what the shifts drop)
+        const unsigned long long K0 = mad_wu(Y >> 1, wh, 9) + hi32(mad_wu(Y >> 1, wl, 0));
+        const long long X = mad_w((int)hi32(K0), ec, mul_w((int)((unsigned)K0 >> 1), ec) >> 31);
+        const unsigned long long K = K0 + (unsigned long long)((X + (X << 1)) >> 21);
+        const int kh = (int)hi32(K), kl = (int)((unsigned)K >> 4);
+        const int gh[6] = {w2.w, w3.x, w3.y, w3.z, w3.w, w4.x}, gl[6] = {w4.y, w4.z, w4.w, w5.x, w5.y, w5.z};
+#pragma unroll
+        for (int y = 0; y < 6; ++y) {
+            I[y] = mad_w(kh, gh[y], I[y]);
+            J[y] = mad_w(kl, gh[y], mad_w(kh, gl[y], J[y]));
+        }
+    }
+    double v[6];
+#pragma unroll
+    for (int x = 0; x < 6; ++x) v[x] = fp64_of(I[x] + ((J[x] + (1 << (kGLow - 1))) >> kGLow), 0);
+    // K 2^(-3/2 m), the limbs and the strength's scale
+    const double gs = odd ? T.gs[1] : T.gs[0];
+    const double sd = __hiloint2double(__double2hiint(gs) + ((((-3 * m) >> 1) + 32 - 147 - kGBits) << 20),
+                                       __double2loint(gs));
+    const double rs = pow2d(T.es);
+    u[0] = fma(fma(rs, v[3], fma(e[2], v[1], -e[1] * v[2])), sd, u[0]);
+    u[1] = fma(fma(rs, v[4], fma(e[0], v[2], -e[2] * v[0])), sd, u[1]);
+    u[2] = fma(fma(rs, v[5], fma(e[1], v[0], -e[0] * v[1])), sd, u[2]);
+}
+
+// ---- geometry ------------------------------------------------------------------------------------------
 
 __device__ __forceinline__ DwTile make_tile(const double c[3], float rho, double gs)
 {
     DwTile t;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        t.c[k] = c[k];
-        if (rho < kInf) words3(c[k], t.c1[k], t.c2[k], t.c3[k]);
-        else t.c1[k] = t.c2[k] = t.c3[k] = 0.0f;
-    }
+    for (int k = 0; k < 3; ++k) t.c[k] = c[k];
+    t.gs[0] = gs;
+    t.gs[1] = gs * 1.4142135623730950488;
     t.rho = rho;
     t.es = exp_above(rho);
-    t.pad = 0.0f;
-    t.gs = gs;
-    t.pad2[0] = t.pad2[1] = 0.0;
     return t;
 }
 
 // Geometry pass of one tile per CTA: q, the far record and the near block.  One thread per node;
 // the radii and the largest strength come from a CTA reduction, so the far records can be written
 // already scaled.  Bound by the FP64 instructions of the stencils; 64-thread CTAs spread small
-// meshes over the SMs (before, 256-thread CTAs: 48 x 48 ran on 9 SMs).
+// meshes over the SMs (with 256-thread CTAs 64 x 64 runs on 16 of them).
 __global__ void __launch_bounds__(kTs)
     geometry_dw_kernel(Geom g, DwMesh m, const double *__restrict__ y, double pref, double grav, double pscale,
                        double gscale, float *__restrict__ near_rec, float *__restrict__ far_rec,
@@ -221,13 +316,11 @@ __global__ void __launch_bounds__(kTs)
     if (!ZM_IDX_OK(pc, g.N) || !ZM_IDX_OK(pcq, g.N)) return;
     double c[3], cq[3], s[3], sq[3];
     double r2 = 0.0, r2q = 0.0;
-    bool ok = true;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         c[k] = y[k * N + pc] * pscale;
         cq[k] = y[k * N + pcq] * pscale;
         const double a = zc[k] * pscale;
-        ok = ok && fabs(a) < 7.0;  // false for NaN
         s[k] = a - c[k];
         sq[k] = a - cq[k];
         r2 = fma(s[k], s[k], r2);
@@ -235,29 +328,23 @@ __global__ void __launch_bounds__(kTs)
     }
     __syncthreads();
     if (valid) {
-        atomicMax(&rmax[0], __float_as_uint(ok ? sqrtf(__double2float_ru(r2)) * 1.000001f : kInf));
-        atomicMax(&rmax[1 + qk], __float_as_uint(ok ? sqrtf(__double2float_ru(r2q)) * 1.000001f : kInf));
+        // not less than kMaxLength (also for NaN): infinite
+        const float rn = sqrtf(__double2float_ru(r2)) * 1.000001f, rq = sqrtf(__double2float_ru(r2q)) * 1.000001f;
+        atomicMax(&rmax[0], __float_as_uint(rn < kMaxLength ? rn : kInf));
+        atomicMax(&rmax[1 + qk], __float_as_uint(rq < kMaxLength ? rq : kInf));
         atomicMax(&gmax, max(hi_abs(gm[0]), max(hi_abs(gm[1]), hi_abs(gm[2]))));
     }
     __syncthreads();
     const int eg = gmax ? (int)(gmax >> 20) - 1022 : 0;  // |strength components| < 2^eg
-    const bool fit = eg >= -400 && eg <= 400 && __uint_as_float(rmax[0]) < 1e30f;
+    const bool fit = eg >= -400 && eg <= 400 && __uint_as_float(rmax[0]) < kInf;
     const double gs = pow2d(fit ? eg : 0) * gscale;
 
     float *fr = far_rec + (size_t)tile * kFarWords;
     float *nf = near_rec + (size_t)tile * kNearWords;
     double *nd = reinterpret_cast<double *>(nf + kFarWords);
-    // zero every column that no node fills
-    if (pt.count < kTs) {
-        for (int e = tid; e < kFarWords; e += kTs)
-            if ((e & (kTs - 1)) >= pt.count) fr[e] = 0.0f;
-        for (int e = tid; e < kFarWords; e += kTs) {
-            const int col = e & (kTs - 1);
-            if ((col & 15) >= quarter_of(pt, col >> 4).count) nf[e] = 0.0f;
-        }
-    }
     if (valid) {
         const int slot = qk * 16 + (li - (qk >> 1) * kSub) * pq.h2 + (lj - (qk & 1) * kSub);
+        if (!ZM_IDX_OK(slot, kTs)) return;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             nd[k * kTs + slot] = zc[k];
@@ -266,128 +353,12 @@ __global__ void __launch_bounds__(kTs)
         if (fit) {
             const double gi = pow2d(-eg);
             const double gg[3] = {gm[0] * gi, gm[1] * gi, gm[2] * gi};
-            put_far(fr + tid, s, gg, exp_above(__uint_as_float(rmax[0])));
-            put_far(nf + slot, sq, gg, exp_above(__uint_as_float(rmax[1 + qk])));
+            put_far(fr + tid * kNodeWords, s, gg, exp_above(__uint_as_float(rmax[0])));
+            put_far(nf + slot * kNodeWords, sq, gg, exp_above(__uint_as_float(rmax[1 + qk])));
         }
     }
     if (tid == 0) info[tile].tile = make_tile(c, fit ? __uint_as_float(rmax[0]) : kInf, gs);
     if (valid && p == pcq) info[tile].quarter[qk] = make_tile(cq, fit ? __uint_as_float(rmax[1 + qk]) : kInf, gs);
-}
-
-__device__ __forceinline__ u64 dup2(float x) { return pk(x, x); }
-__device__ __forceinline__ u64 rsq2(u64 v) { return pk(dev::rsqrt_approx(lane0(v)), dev::rsqrt_approx(lane1(v))); }
-
-// acc += a b, 64-bit; as PTX because the C expression compiles to three instructions (counted: 13
-// instead of 4 integer multiplies for 4 products)
-__device__ __forceinline__ void mad_wide(long long &acc, int a, int b)
-{
-    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
-}
-
-// The far pairs of one target and one source tile (record in shared memory): adds sum_j K (s - t) x g
-// to u.  td: the target, scaled, in FP64; tw: its words.
-__device__ __forceinline__ void far_tile(const float *__restrict__ rec, int groups, const double td[3],
-                                           const float *tw, const DwTile &T, double d2, float d2f, double u[3])
-{
-    df t[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        // exact word differences; the leading one is zero or larger than the second
-        const df h = fast_two_sum(__fsub_rn(tw[k], T.c1[k]), __fsub_rn(tw[3 + k], T.c2[k]));
-        t[k] = fast_two_sum(h.hi, __fadd_rn(h.lo, __fsub_rn(tw[6 + k], T.c3[k])));
-    }
-    const double ex = td[0] - T.c[0], ey = td[1] - T.c[1], ez = td[2] - T.c[2];
-    const double t2d = fma(ex, ex, fma(ey, ey, ez * ez)), B = t2d + d2;
-    // B + C with the power of two C above B: the leading part, rounded to C's grid, from B's leading 23
-    // mantissa bits, and the signed rest from its last 30 (no FP64 instructions)
-    const int bhi = __double2hiint(B), eq = (bhi >> 20) - 1022;
-    const unsigned blo = (unsigned)__double2loint(B);
-    const u64 CC = dup2(__int_as_float((127 + eq) << 23));
-    const u64 F0 = dup2(__int_as_float(((127 + eq) << 23) + (1 << 22) + (((bhi & 0xfffff) << 2) | (blo >> 30)) +
-                                       ((blo >> 29) & 1)));
-    const u64 BL = dup2(__fmul_rn(__int2float_rn((int)(blo << 2) >> 2), __int_as_float((127 + eq - 53) << 23)));
-    u64 mh[3], ml[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        mh[k] = dup2(-2.0f * t[k].hi);
-        ml[k] = dup2(-2.0f * t[k].lo);
-    }
-    // the largest K of the tile gives the scale: K 2^S < 2^30
-    const float t2 = fmaf(t[0].hi, t[0].hi, fmaf(t[1].hi, t[1].hi, t[2].hi * t[2].hi));
-    const float tm = __fsub_rn(__fmul_rn(t2, dev::rsqrt_approx(t2)), T.rho);
-    const float ym = dev::rsqrt_approx(__fmaf_rn(tm, tm, d2f));
-    const float km = __fmul_rn(__fmul_rn(__fmul_rn(ym, ym), ym), 1.001f);
-    const int S = 29 - ((int)(__float_as_uint(km) >> 23) - 127);
-    const u64 sc = dup2(__uint_as_float((unsigned)(127 + S) << 23));
-
-    const u64 kOne = dup2(1.0f), kC1 = dup2(1.5f), kC2 = dup2(1.875f);
-    const u64 kMagic = dup2(12582912.0f);
-    long long I[6] = {0, 0, 0, 0, 0, 0};
-    u64 al[6] = {0, 0, 0, 0, 0, 0};
-    const ulonglong2 *r4 = reinterpret_cast<const ulonglong2 *>(rec);  // four sources of row k: r4[k * 16 + g]
-    constexpr int H = kTs / 4;
-#pragma unroll 1
-    for (int gq = 0; gq < groups; ++gq) {
-        const ulonglong2 *r = r4 + gq;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            auto row = [&](int k) {
-                const ulonglong2 v = r[k * H];
-                return h ? v.y : v.x;
-            };
-            const u64 ah = row(kRowA), alo = row(kRowA + 1);
-            u64 f = add2(F0, ah);
-            u64 l = add2(add2(BL, alo), sub2(ah, sub2(f, F0)));
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const u64 sh = row(k), sl = row(3 + k);
-                const u64 f1 = fma2(mh[k], sh, f);
-                const u64 er = fma2(mh[k], sh, sub2(f, f1));  // m s - (f1 - f), exact
-                l = add2(l, er);
-                l = fma2(mh[k], sl, l);
-                l = fma2(ml[k], sh, l);
-                f = f1;
-            }
-            const u64 qh = sub2(f, CC), nq = sub2(CC, f);
-            const u64 y = rsq2(qh);
-            const u64 w = mul2(y, y), nw = neg2(w);
-            const u64 wl = fma2(y, y, nw);
-            u64 e = fma2(nq, w, kOne);
-            e = fma2(nq, wl, e);
-            e = fma2(l, nw, e);
-            const u64 ys = mul2(y, sc);
-            const u64 kh = mul2(w, ys);
-            u64 kl = fma2(wl, ys, fma2(w, ys, neg2(kh)));
-            const u64 c = mul2(fma2(e, kC2, kC1), e);
-            kl = fma2(kl, c, kl);
-            kl = fma2(kh, c, kl);
-            // integer part of kl into the integer K, the rest below half a unit
-            const u64 km2 = add2(kl, kMagic);
-            kl = sub2(kl, sub2(km2, kMagic));
-            const int ka = __float2int_rn(lane0(kh)) + ((int)(unsigned)km2 - 0x4b400000);
-            const int kb = __float2int_rn(lane1(kh)) + ((int)(unsigned)(km2 >> 32) - 0x4b400000);
-#pragma unroll
-            for (int x = 0; x < 6; ++x) {
-                const u64 gi = row(kRowI + x);
-                mad_wide(I[x], ka, (int)(unsigned)gi);
-                mad_wide(I[x], kb, (int)(unsigned)(gi >> 32));
-                al[x] = fma2(kh, row(kRowR + x), al[x]);
-                al[x] = fma2(kl, row(kRowF + x), al[x]);
-            }
-        }
-    }
-    // the remainders into the integers (below 2^10 K units, to 2^-20), then the tile's sums in FP64
-    double v[6];
-#pragma unroll
-    for (int x = 0; x < 6; ++x) {
-        const int rest = __float2int_rn(__fmul_rn(__fadd_rn(lane0(al[x]), lane1(al[x])), 1048576.0f));
-        v[x] = (double)(I[x] + ((long long)rest << (kGBits - 20)));
-    }
-    const double sd = __hiloint2double(__double2hiint(T.gs) - ((S + kGBits) << 20), __double2loint(T.gs));
-    const double rs = pow2d(T.es);
-    u[0] = fma(fma(rs, v[3], fma(ez, v[1], -ey * v[2])), sd, u[0]);
-    u[1] = fma(fma(rs, v[4], fma(ex, v[2], -ez * v[0])), sd, u[1]);
-    u[2] = fma(fma(rs, v[5], fma(ey, v[0], -ex * v[1])), sd, u[2]);
 }
 
 struct DwArgs {
@@ -404,18 +375,16 @@ struct DwArgs {
     int *err;
 };
 
-// Distance between the centre words of a tile and a point's, less the point's own radius.
-__device__ __forceinline__ float gap(const DwTile &s, const float *w, float rho)
+// Distance between a tile's centre and a point, less the point's own radius.
+__device__ __forceinline__ float gap(const DwTile &s, const double *p, float rho)
 {
-    const float dx = (s.c1[0] - w[0]) + (s.c2[0] - w[3]);
-    const float dy = (s.c1[1] - w[1]) + (s.c2[1] - w[4]);
-    const float dz = (s.c1[2] - w[2]) + (s.c2[2] - w[5]);
+    const float dx = (float)(s.c[0] - p[0]), dy = (float)(s.c[1] - p[1]), dz = (float)(s.c[2] - p[2]);
     return sqrtf(dx * dx + dy * dy + dz * dz) * 0.9999f - rho;
 }
-// 2^-20 keeps K in range; an infinite radius is never far.
+// 2^-20 and 2^20 keep K and the scale factors in range; an infinite radius is never far.
 __device__ __forceinline__ bool is_far(float gap, float kappa, float rho)
 {
-    return gap >= kappa * rho && gap >= 9.5367431640625e-7f;
+    return gap >= kappa * rho && gap >= 1.0f / kMaxLength && gap <= kMaxLength;
 }
 
 __global__ void __launch_bounds__(kTs, 7) brdw_kernel(const DwArgs a)
@@ -433,21 +402,14 @@ __global__ void __launch_bounds__(kTs, 7) brdw_kernel(const DwArgs a)
     if (!ZM_IDX_OK(p, N)) return;
     const double tx = a.z[p], ty = a.z[N + p], tz = a.z[2 * N + p];
     const double td[3] = {tx * a.pscale, ty * a.pscale, tz * a.pscale};
-    float tw[9];
-    words3(td[0], tw[0], tw[3], tw[6]);
-    words3(td[1], tw[1], tw[4], tw[7]);
-    words3(td[2], tw[2], tw[5], tw[8]);
     // the target tile's sphere, and the sphere of this warp's 32 targets around one of them
-    float cw[6], ct[6];
     const DwTile me = a.info[tt].tile;
+    double cw[3];
     float wr = 0.0f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        ct[k] = me.c1[k];
-        ct[3 + k] = me.c2[k];
-        cw[k] = __shfl_sync(0xffffffffu, tw[k], 20);
-        cw[3 + k] = __shfl_sync(0xffffffffu, tw[3 + k], 20);
-        const float d = (tw[k] - cw[k]) + (tw[3 + k] - cw[3 + k]);
+        cw[k] = __shfl_sync(0xffffffffu, td[k], 20);
+        const float d = (float)(td[k] - cw[k]);
         wr = fmaf(d, d, wr);
     }
     wr = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(sqrtf(wr) * 1.0001f)));
@@ -470,7 +432,7 @@ __global__ void __launch_bounds__(kTs, 7) brdw_kernel(const DwArgs a)
         bool far = false;
         if (tid < n && ZM_IDX_OK(tile_of(tid), a.ntiles)) {
             const DwTile &s = a.info[tile_of(tid)].tile;
-            far = is_far(gap(s, ct, me.rho), a.kappa, s.rho);
+            far = is_far(gap(s, me.c, me.rho), a.kappa, s.rho);
         }
         const uint32_t mk = __ballot_sync(0xffffffffu, far);
         if ((tid & 31) == 0) farmask[tid >> 5] = mk;
@@ -500,7 +462,7 @@ __global__ void __launch_bounds__(kTs, 7) brdw_kernel(const DwArgs a)
                     if (count == 0) continue;
                     const DwTile s = whole ? I.tile : I.quarter[q];
                     if (whole || is_far(gap(s, cw, wr), a.kappa, s.rho)) {
-                        far_tile(stage[b] + 16 * q, (count + 3) >> 2, td, tw, s, a.d2s, (float)a.d2s, u);
+                        far_tile(stage[b] + 16 * kNodeWords * q, count, td, s, a.d2s, (float)a.d2s, u);
                         continue;
                     }
                     const double *r = reinterpret_cast<const double *>(stage[b] + kFarWords) + 16 * q;
@@ -547,17 +509,15 @@ __global__ void __launch_bounds__(kTs, 7) brdw_kernel(const DwArgs a)
 
 int length_exponent(const Geom &g) { return std::ilogb(std::max(g.L1, g.L2)); }
 
-// Factor of the far classification: 2 source radii, or 3 on small meshes, whose plain FP64 sums are
-// short and round little (u at 64 x 64 against long double: 5.2e-16 with 3, 7.3e-16 with 2, 7.5e-16
-// for the plain sum; 0.27 and 0.24 ms).  Lengths or a core size outside the FP32-pair range leave
-// every pair near.
+// Factor of the far classification.  Lengths or a core size outside the range of the integers' scales
+// leave every pair near.
 float kappa_of(const zm_ctx *c)
 {
     const Geom &g = c->geom;
     const int e = length_exponent(g);
     const double d = std::ldexp(c->delta, -e);
     if (e < -100 || e > 100 || !(d < 16.0) || !(std::min(g.L1, g.L2) > 0)) return kInf;
-    return g.N >= 96 * 96 ? 2.0f : 3.0f;
+    return kKappa;
 }
 
 DwMesh dw_mesh(const Geom &g)
@@ -567,8 +527,10 @@ DwMesh dw_mesh(const Geom &g)
 
 }  // namespace
 
-// Meshes below 56^2 keep the plain FP64 kernel: most of their tiles are near each other, and its short
-// sums are the more accurate ones (48 x 48: 0.31 against 0.25 ms, 3.5e-16 against 4.5e-16).
+// Meshes below 56^2 keep the plain FP64 kernel.  One evaluation, plain / here, and the errors of u: 32 x 32
+// 0.090 / 0.106 ms, 2.0e-16 / 2.4e-16; 40 x 40 0.190 / 0.132 ms, 3.2e-16 / 2.6e-16; 48 x 48 0.305 / 0.196 ms,
+// 3.5e-16 / 2.2e-16; 56 x 56 0.610 / 0.227 ms, 5.1e-16 / 2.0e-16.  (The line lies where a less accurate far form,
+// FP32 pairs, began to be the better one; the present form would be from 40^2 on.)
 constexpr int kDwMinN = 56 * 56;
 
 bool brdw_mesh(const Geom &g) { return g.N >= kDwMinN; }
