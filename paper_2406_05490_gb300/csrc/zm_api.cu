@@ -1,6 +1,8 @@
 // zm_api.cu -- the C ABI of libzm.so (declared and documented in include/zm.h): context
 // lifecycle, argument checks, host/device pointer handling, and the orchestration of one
 // derivative evaluation (paper Sec. 3.1 ZModel) and of SSP-RK3 steps (Sec. 3.1 TimeIntegrator).
+#include <cuda.h>
+
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -145,18 +147,53 @@ static bool is_device_ptr(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Whether the context's kernels can read or write p directly: managed memory or memory of the context's
-// own GPU, aligned to its type.
-static bool kernel_ptr(const zm_ctx *c, const double *p)
+// How the context's kernels may use a caller's array of `count` doubles.
+enum Access {
+    kByCopy,    // by a staging copy: host memory, another GPU's, or not aligned to its type
+    kDirect,    // in place: managed memory or memory of the context's own GPU, all in one allocation
+    kTooShort,  // not at all: it runs past its allocation into memory that is not mapped (a copy would be
+                // refused; a kernel would fault)
+};
+static Access access_of(const zm_ctx *c, const double *p, size_t count)
 {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return kByCopy;
     }
-    return (a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == c->device)) &&
-           reinterpret_cast<uintptr_t>(p) % sizeof(double) == 0;
+    if ((a.type != cudaMemoryTypeManaged && (a.type != cudaMemoryTypeDevice || a.device != c->device)) ||
+        reinterpret_cast<uintptr_t>(p) % sizeof(double) != 0)
+        return kByCopy;
+    using RangeFn = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const RangeFn range_of = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<RangeFn>(f);
+    }();
+    if (!range_of) return kByCopy;
+    const CUdeviceptr first = reinterpret_cast<CUdeviceptr>(p), end = first + count * sizeof(double);
+    for (CUdeviceptr at = first; at < end;) {
+        CUdeviceptr base = 0;
+        size_t size = 0;
+        if (range_of(&base, &size, at) != CUDA_SUCCESS || base + size <= at) return at == first ? kByCopy : kTooShort;
+        if (base + size >= end) return at == first ? kDirect : kByCopy;
+        at = base + size;
+    }
+    return kByCopy;
 }
+// The same for z (3N) and w (2N) together; either may be null.
+static Access access_of_state(const zm_ctx *c, const double *z, const double *w)
+{
+    const size_t N = c->geom.N;
+    const Access az = z ? access_of(c, z, 3 * N) : kDirect, aw = w ? access_of(c, w, 2 * N) : kDirect;
+    return az == kTooShort || aw == kTooShort ? kTooShort : az == kDirect && aw == kDirect ? kDirect : kByCopy;
+}
+static int too_short() { return set_error(ZM_ERR_CUDA, "a device array runs past the end of its allocation"); }
 
 static int copy_in(zm_ctx *c, double *dst, const double *src, size_t count)
 {
@@ -380,7 +417,9 @@ int zm_set_state(zm_ctx *c, const double *z, const double *w)
 {
     if (!c || !z || !w) return set_error(ZM_ERR_INVALID, "zm_set_state: null argument");
     const size_t N = c->geom.N;
-    if (c->df64 && kernel_ptr(c, z) && kernel_ptr(c, w)) return df_state_in(c, z, w, c->y0);
+    const Access access = c->df64 ? access_of_state(c, z, w) : kByCopy;
+    if (access == kTooShort) return too_short();
+    if (access == kDirect) return df_state_in(c, z, w, c->y0);
     double *dst = c->df64 ? c->yb : c->y0;  // double word: stage FP64 in yb, convert into y0
     int rc = copy_in(c, dst, z, 3 * N);
     if (!rc) rc = copy_in(c, dst + 3 * N, w, 2 * N);
@@ -397,7 +436,9 @@ int zm_get_state(zm_ctx *c, double *z, double *w)
     bool host = false;
     int rc = ZM_OK;
     const double *src = c->y0;
-    if (c->df64 && (!z || kernel_ptr(c, z)) && (!w || kernel_ptr(c, w))) return df_state_out(c, c->y0, z, w);
+    const Access access = c->df64 ? access_of_state(c, z, w) : kByCopy;
+    if (access == kTooShort) return too_short();
+    if (access == kDirect) return df_state_out(c, c->y0, z, w);
     if (c->df64) {  // FP64 copy of the state in yb (a stage buffer, free between calls)
         rc = df_convert(c, c->y0, c->yb, 5 * N, 1, 0);
         src = c->yb;
@@ -417,7 +458,9 @@ int zm_velocity(zm_ctx *c, const double *z, const double *w, double *u, double *
     const size_t N = c->geom.N;
     const double *y = c->y0;
     int rc = ZM_OK;
-    if (z && c->df64 && kernel_ptr(c, z) && kernel_ptr(c, w)) {
+    const Access access = z && c->df64 ? access_of_state(c, z, w) : kByCopy;
+    if (access == kTooShort) return too_short();
+    if (access == kDirect) {
         rc = df_state_in(c, z, w, c->ya);
         y = c->ya;
     } else if (z) {
