@@ -25,8 +25,8 @@
 // ms per evaluation, FP64 butterflies / integers: 1024^2 0.452 / 0.102, 4096^2 6.85 / 1.44, 4864^2 13.18 /
 // 2.88, 512^2 0.115 / 0.052, 152 x 304 0.138 / 0.064, 128^2 0.031 / 0.029 (latency).  Relative error of u
 // against a long double transform: 128^2 3.8e-16 / 3.2e-16, 256^2 4.7e-16 / 4.3e-16, 512^2 5.6e-16 /
-// 5.2e-16, 152 x 304 5.5e-16 / 5.3e-16, 608 x 152 5.5e-16 / 5.6e-16.  What bounds it now: latency at 16 warps per SM (128 registers for 16 values), the schedulers
-// issuing in 34 to 47 % of cycles.
+// 5.2e-16, 152 x 304 5.5e-16 / 5.3e-16, 608 x 152 5.5e-16 / 5.6e-16.  What bounds it now: latency at 16
+// warps per SM (128 registers for 16 values), the schedulers issuing in 34 to 47 % of cycles.
 //
 // Sides L = R M with M = 2^a (a >= 3) and R odd (3 .. 19; 4864 = 19 x 256 is the paper's
 // low-order mesh, Sec. 5.1) add one radix-R stage: before the length-M transforms in decimation
@@ -475,6 +475,12 @@ __device__ __forceinline__ void clear_words(unsigned *words, int count)
     __syncthreads();
 }
 
+// The leading word of |v|, at least 1 where v is not zero (denormal numbers have theirs in the other).
+__device__ __forceinline__ unsigned size_bits(double v)
+{
+    return ((unsigned)__double2hiint(v) & 0x7fffffffu) | (__double2loint(v) != 0 ? 1u : 0u);
+}
+
 // pass A: rows i of length n2 from w1 + i w2; forward; write out[j][i] (transposed).
 template <int A, bool kMix>
 __global__ void __launch_bounds__(threads_for(A, kMix), minb_for(A, kMix))
@@ -503,7 +509,7 @@ __global__ void __launch_bounds__(threads_for(A, kMix), minb_for(A, kMix))
         for (int k = 0; k < kBatch; ++k) {
             const int e = e0 + k * blockDim.x;
             if (e < total) {
-                mx = max(mx, max((unsigned)__double2hiint(a[k]) & 0x7fffffffu, (unsigned)__double2hiint(b[k]) & 0x7fffffffu));
+                mx = max(mx, max(size_bits(a[k]), size_bits(b[k])));
                 sx[phys(e)] = make_ulonglong2((unsigned long long)__double_as_longlong(a[k]),
                                               (unsigned long long)__double_as_longlong(b[k]));
             }
@@ -514,8 +520,8 @@ __global__ void __launch_bounds__(threads_for(A, kMix), minb_for(A, kMix))
     if ((threadIdx.x & 31) == 0) atomicMax(&words[0], mx);
     __syncthreads();
     mx = words[0];
-    // |w| < 2^eb; to integers below 2^54
-    const int eb = max((int)(mx >> 20) - 1022, -940);
+    // |w| < 2^eb (denormal numbers: the least exponent); to integers below 2^54
+    const int eb = max((int)(mx >> 20) - 1022, -1021);
     unsigned o = 0;
     for (int e = threadIdx.x; e < rows * L; e += blockDim.x) {  // the thread's own elements
         const ulonglong2 v = sx[phys(e)];

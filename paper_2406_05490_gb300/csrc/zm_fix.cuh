@@ -83,7 +83,7 @@ __device__ __forceinline__ Shift make_shift(int s)
 // Between FP64 words and fixed point without the FP64 pipe, which the conversions and their scale factors
 // would hold longer than the first and last pass can hide (1024 x 1024: pass A 30.8 -> 25.8 us, pass C 42.0 ->
 // 37.7; 4096 x 4096: 403 -> 395 and 429 -> 431).
-// round(v 2^(54 - eb)) of an FP64 number below 2^eb (eb >= -940), from its bits; ties away from zero.
+// round(v 2^(54 - eb)) of an FP64 number below 2^eb (eb >= -1021), from its bits; ties away from zero.
 __device__ __forceinline__ long long fix_of(unsigned long long v, int eb)
 {
     const int e = (int)(v >> 52) & 0x7ff;
