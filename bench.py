@@ -9,7 +9,7 @@ A = 0.5, g = 1, delta = 0.1 dx, dt = 1e-3) with FP32-compensated Birkhoff-Rott p
 Each step evaluates 3 x 65536^2 = 1.29e10 pair interactions.
 
 Also measured and reported beside the headline (not the headline):
-  * the plain FP64 form of the same step (the comparator);
+  * the same step in FP64 (the comparator; its far pairs are evaluated in integers);
   * the low-order 1024 x 1024 FFT Riesz step (8 modes, amplitude 0.02, A = 0.7);
   * the 32 x 32 single-mode FP64 step (launch bound).
 
@@ -487,7 +487,7 @@ def bench_low_order(zm, torch, inputs, flush, nl, steps, warmup, df64, fp64_tflo
 def bench_batched(zm, torch, inputs, flush, steps=10, warmup=2, count=64):
     """64 periodic interfaces, sides log-uniform in [64, 384] (seed 0), 4 modes, A ~ U[0.2, 0.8],
     FP32C, one graph-replayed RK3 step per timed step; beside it the same interfaces solved one at
-    a time (FP32C contexts) and the plain per-instance FP64 form on a sample of them."""
+    a time (FP32C contexts) and the per-instance FP64 form on a sample of them."""
     insts = inputs.ragged_batch(count=count, lo=64, hi=384, n_modes=4, seed=0)
     meshes = [(r.n, r.n, 1.0, 1.0, True) for r in insts]
     h = zm.zm_batch_create(meshes, [r.atwood for r in insts], g=1.0, delta=[0.1 / r.n for r in insts])
@@ -540,7 +540,7 @@ def bench_batched(zm, torch, inputs, flush, steps=10, warmup=2, count=64):
     for m in models:
         m.close()
     out["one_at_a_time_fp32c_gpairs_per_s"] = pairs_step / (t_ms * 1e-3) / 1e9
-    # plain per-instance FP64 form on a sample (the smallest, a median and the largest side)
+    # per-instance FP64 form on a sample (the smallest, a median and the largest side)
     order = sorted(range(count), key=lambda k: insts[k].n)
     sample = [order[0], order[count // 2], order[-1]]
     f_pairs, f_ms = 0, 0.0
@@ -627,7 +627,7 @@ def serve_trace(zm, trace, budget, slots, dt=1e-3, policy=None, cap=0):
 
 
 def fp64_sequential_trace(zm, trace, dt=1e-3):
-    """The plain per-instance FP64 form as a server: one request at a time in arrival order,
+    """The per-instance FP64 form as a server: one request at a time in arrival order,
     each on its own FP64 context; latency = completion - arrival."""
     import numpy as np
     t0 = time.perf_counter()
@@ -650,7 +650,7 @@ def fp64_sequential_trace(zm, trace, dt=1e-3):
 
 
 def fp64_service_model(zm, inputs, sides=(32, 64, 128, 192, 256), dt=1e-3):
-    """Measured service time of one request in the plain per-instance FP64 form (context
+    """Measured service time of one request in the per-instance FP64 form (context
     creation, state upload, one RK3 step, state download, teardown), per mesh side; fitted as
     t(n) = a + b * 3 n^4 (fixed cost plus pair interactions) for the queue model below."""
     import numpy as np
@@ -676,7 +676,7 @@ def fp64_service_model(zm, inputs, sides=(32, 64, 128, 192, 256), dt=1e-3):
 
 
 def fp64_queue_model(model, trace):
-    """Latencies of the plain per-instance FP64 form serving `trace` one request at a time in
+    """Latencies of the per-instance FP64 form serving `trace` one request at a time in
     arrival order (a single FIFO server), from the measured service times: request k starts at
     max(arrival, previous completion) and takes nsteps * (a + b * 3 n^4)."""
     import numpy as np
@@ -697,9 +697,9 @@ SERVE_CAP = 20_000_000_000  # SRPT: pair interactions per server iteration (abou
 def bench_serving(zm, inputs, count=256, budget=16 << 30, slots=64, compare=False):
     """Poisson arrivals at 200/s, sides log-uniform in [32, 512], 20 RK3 steps each (FP32C),
     256 requests, served shortest-remaining-work-first; then a trace of the same kind at about
-    70% of the measured capacity; the plain per-instance FP64 form on that same trace (modelled
+    70% of the measured capacity; the per-instance FP64 form on that same trace (modelled
     from its measured service times: run for real it would take over an hour); and a reduced
-    trace (sides [32, 96], 5 steps) served both by the server and, for real, by the plain FP64
+    trace (sides [32, 96], 5 steps) served both by the server and, for real, by the FP64
     form.  compare=True adds the first-come-first-served all-resident policy on both traces."""
     full = inputs.poisson_trace(count=count, rate_hz=200.0, lo=32, hi=512, nsteps=20, seed=0)
     out = {"offered": serve_trace(zm, full, budget, slots, policy=zm.ZM_SERVE_SRPT, cap=SERVE_CAP)}
@@ -800,7 +800,7 @@ def run_gb300(args):
 
     extras = {}
     if not args.no_extras:
-        # plain FP64 comparator: the same interface, FP64 pair terms
+        # FP64 comparator: the same interface
         m64 = zm.ZModel(n, periodic=True, atwood=0.5, g=1.0, delta=0.1 / n, fp32c=False)
         # the headline's FP32C derivative against the FP64 path on the same interface with
         # vorticity (w = 0 makes the velocity vanish), per field: the accuracy side of the
@@ -816,7 +816,7 @@ def run_gb300(args):
         k64 = 2
         ms64, prof64 = timed_steps(m64, zm, torch, k64, 1, flush)
         m64.close()
-        # its all-pairs kernel: near pairs in FP64, far ones in FP32 pairs and integers; the share of
+        # its all-pairs kernel: near pairs in FP64, far ones in 64-bit integers; the share of
         # the FP64 pipe from the counted FP64 instructions and the rate of a probe kernel
         br64_ms = prof64["ms"]["br"] / max(prof64["launches"]["br"], 1)
         fp64_peak = max(zm.zm_measure_peak(zm.PEAK_FP64) for _ in range(3)) / 1e12
@@ -824,7 +824,7 @@ def run_gb300(args):
         extras["fp64_plain"] = {"gpairs_per_s": pairs_per_step * k64 / (ms64 * 1e-3) / 1e9,
                                 "steps_per_s": k64 / (ms64 * 1e-3), "ms_per_step": ms64 / k64,
                                 "steps": k64,
-                                "roofline": {"bound": "fma pipe (far pairs in FP32 pairs), fp64 pipe (near pairs)",
+                                "roofline": {"bound": "integer multiply and ALU pipes (far pairs), fp64 pipe (near pairs)",
                                              "fp64_peak": fp64_peak, "unit": "TFLOP/s",
                                              "peak_basis": "measured FP64 FMA probe (zm_measure_peak)",
                                              "br_ms_per_launch": br64_ms,

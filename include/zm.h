@@ -62,7 +62,10 @@ extern "C" {
 #define ZM_ORDER_LOW 0
 #define ZM_ORDER_MEDIUM 1
 #define ZM_ORDER_HIGH 2
-#define ZM_PREC_FP64 0x000
+#define ZM_PREC_FP64 0x000  /* every result to FP64 precision: FP64 instructions, or integers of
+                               54 to 64 bits where the FP64 pipe would bound the time (the FFT;
+                               from 56^2 nodes on, Birkhoff-Rott pairs that are far apart
+                               compared with their source tile) */
 #define ZM_PREC_FP32C 0x100 /* BR pair terms in FP32 (hi/lo positions near, tile-local
                                coordinates far), per-tile FP32 partials, exact 64-bit fixed-point
                                accumulation across tiles (finer than FP64); all else FP64 */
@@ -360,11 +363,13 @@ void zm_server_destroy(zm_server *s);
 /* The paper has no counterpart: this entry point exists for callers that cannot allocate GPU
  * memory -- a host application that reserves all device memory at start-up and forbids later
  * allocations, or code that must not pay the device-wide synchronisation that cudaMalloc and
- * cudaFree imply.  It computes the FP64 all-pairs sum of zm_velocity's high-order path on
- * caller-prepared inputs and allocates nothing: no cudaMalloc, cudaFree or allocating library
- * call.  Its workspace (tile-major source records, split partial sums, a status word; 9 MiB in
- * all) is one static device array inside libzm.so, held by every GPU that loads the library
- * until the process exits.
+ * cudaFree imply.  It computes the all-pairs sum of the high-order velocity with every pair in
+ * FP64 instructions, as zm_velocity does below 56^2 nodes only (at 256^2 nodes this takes about
+ * nine times as long as zm_velocity, whose far pairs are in integers), on caller-prepared
+ * inputs, and allocates nothing: no cudaMalloc, cudaFree or allocating library call.  Its
+ * workspace (tile-major source records, split partial sums, a status word; 9 MiB in all) is one
+ * static device array inside libzm.so, held by every GPU that loads the library until the
+ * process exits.
  *
  *   u_i = sum_j (z_j - z_i) x gamma_j / (|z_j - z_i|^2 + delta^2)^(3/2),  i, j < n
  *

@@ -6,9 +6,10 @@
 // What bounds it.  GB300 executes 2 FP64 instructions per clock and SM, so the 21 FP64 instructions of
 // a pair (zm_br.cu) cost 10.5 clocks of an SM whose other pipes idle (measured: the pipe 90 % busy, 190 ms
 // per 256 x 256 evaluation).  A pair far apart compared with its source tile is evaluated here in 64-bit
-// integers instead, to the same precision: 29 integer multiply-adds 32 x 32 + 64 bits (about 30 per clock
-// and SM), some 50 other integer operations, 9 in FP32, one reciprocal square root: 1.5 clocks, the
-// multiply and ALU pipes 61 and 53 % busy, the FP64 pipe 19 %, the schedulers issuing in 54 % of cycles.
+// integers instead, to the same precision: 29 integer multiply-adds 32 x 32 + 64 bits (60 per clock and
+// SM), some 50 other integer operations, 9 in FP32, one reciprocal square root, 108 instructions with the
+// rest: 1.6 clocks, the multiply and ALU pipes 61 and 53 % busy, the FP64 pipe 19 %, the schedulers issuing
+// in 54 % of cycles.
 // 190.3 -> 21.4 ms at 256 x 256, 13.0 -> 1.63 at 128 x 128, 7.5 -> 0.93 at 90 x 131, 0.81 -> 0.23 at
 // 64 x 64 (one evaluation).  (q and K as FP32 pairs take 12.5 ms at 256 x 256 but hold a far pair to 2^-46
 // only: u is then 2e-14 off, relative, where all strength lies further away than the near tiles.)

@@ -216,7 +216,7 @@ Tiling make_tiling(const Geom &g);  // 16 x 16 patches
 Tiling make_tiling_shape(const Geom &g, int tp1, int tp2);
 int launch_br(zm_ctx *c, const double *y);  // FP64 path (then launch_reduce)
 
-// ---- the same for meshes of at least 48^2 nodes: far pairs in FP32 pairs (zm_brdw.cu) --------------
+// ---- the same for meshes of at least 56^2 nodes: far pairs in 64-bit integers (zm_brdw.cu) ---------
 bool brdw_mesh(const Geom &g);
 BrPlan plan_brdw(const Geom &g, int sm_count);
 size_t brdw_near_bytes(const Geom &g);
